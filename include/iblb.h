@@ -348,19 +348,11 @@ int ibl_regularize_now(ibl_mesh *m, int *iters);
  * int32, one-ring neighbours as returned by ibl_copy_neighbours), and
  * result (2 int32: iterations, 1 if converged else 0).  Asynchronous on
  * `stream` (a cudaStream_t, NULL = legacy default stream).
- * Scratch: a fixed array inside the library (16384 nodes x 9 doubles,
- * 1.18 MB) that every GPU loading the library holds until the process
- * exits; n_nodes above 16384 is rejected with IBL_EINVAL.  The first call
- * on a device looks up that array's device address (with the caller's
- * current device), so make the first call on each device before any stream
- * capture.  The address is looked up again whenever the calling thread's
- * current context is not the one it was looked up in (a driver-API context
- * made current, or the primary context created anew after
- * cudaDeviceReset): make the first call after such a change outside a
- * stream capture too.  Every call uses the same array and leaves its contents behind;
- * each call writes every element it reads first, so nothing needs
- * clearing, but calls whose executions overlap on the GPU (other streams,
- * other threads) race on it.  Calls no allocating routine. */
+ * Scratch: the shared memory of one thread-block cluster; n_nodes above
+ * 16384 is rejected with IBL_EINVAL.  No device memory is held between calls,
+ * and calls on different buffers may overlap.  Make the first call on each
+ * device outside a stream capture (it asks the device for its cluster
+ * sizes).  Calls no allocating routine. */
 int ibl_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes, double alpha,
                            double gamma, double tol, int max_iter, int plus_sign, int32_t *result, void *stream);
 

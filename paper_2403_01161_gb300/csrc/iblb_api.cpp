@@ -951,20 +951,21 @@ int ensemble_one_step(ibl_ensemble *e, cudaStream_t sL, cudaStream_t sH)
     err = iblb::launch_ensemble_interp(e->v, sH, e->hi_prio);
     if (err != cudaSuccess) return cuda_fail(err, "ensemble interpolation launch");
     bool reg = false, obs = false;
-    for (ibl_lb *lb : e->m) {
-        ibl_mesh *mm = lb->mesh;
-        if (mm->reg_every > 0 && next % mm->reg_every == 0) {
-            // rewrites the member's patch of the next step: the next outside update waits for it
-            err = iblb::launch_regularize(lb->v, mm->v, mm->reg, (int)(next % 3), sH, e->hi_prio);
-            if (err != cudaSuccess) return cuda_fail(err, "ensemble regularisation launch");
-            reg = true;
-        }
+    std::vector<char> due(e->m.size(), 0);
+    std::vector<iblb::RegParams> params(e->m.size());
+    for (size_t k = 0; k < e->m.size(); ++k) {
+        const ibl_mesh *mm = e->m[k]->mesh;
+        due[k] = mm->reg_every > 0 && next % mm->reg_every == 0;
+        params[k] = mm->reg;
+        reg = reg || due[k];
     }
     if (reg) {
+        // rewrites the members' patches of the next step: the next outside update waits for it
+        err = iblb::launch_regularize_batched(e->v, due, params, (int)(next % 3), sH, e->hi_prio);
+        if (err != cudaSuccess) return cuda_fail(err, "ensemble regularisation launch");
         err = cudaEventRecord(evNear[par], sH);
         if (err != cudaSuccess) return cuda_fail(err, "ensemble event");
     }
-    std::vector<char> due(e->m.size(), 0);
     for (size_t k = 0; k < e->m.size(); ++k) {
         const ibl_mesh *mm = e->m[k]->mesh;
         due[k] = mm->readout_every > 0 && next % mm->readout_every == 0;

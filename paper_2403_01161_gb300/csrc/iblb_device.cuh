@@ -430,6 +430,65 @@ __device__ double block_max(double v, double *sh)
     return out;
 }
 
+// Patch of lattice nodes the droplet's stencils can touch, from the node
+// bounding box [mn, mx]: floor(mn)-1 .. floor(mx)+2 per axis (periodic axes
+// keep the lower corner inside the box and may wrap; Zou-He axes clamp).
+// `grow` extra nodes on each side (1 covers the nodes' motion over one more
+// step: |u| <= 0.3 keeps floor(r) within one node).
+__device__ void write_patch(const LbView &L, const double mn[3], const double mx[3], int buf, int grow)
+{
+    for (int a = 0; a < 3; ++a) {
+        const int n = L.n[a];
+        double lo_d = mn[a], hi_d = mx[a];
+        if (!(lo_d > -1e8 && lo_d < 1e8) || !(hi_d > -1e8 && hi_d < 1e8) || hi_d < lo_d) {
+            L.ctl->patch_lo[buf][a] = 0;
+            L.ctl->patch_ext[buf][a] = n - 1;
+            continue;
+        }
+        long long lo = (long long)floor(lo_d) - 1 - grow, hi = (long long)floor(hi_d) + 2 + grow;
+        if (L.bc[a] == IBL_BC_PERIODIC) {
+            if (hi - lo + 1 >= n) {
+                lo = 0;
+                hi = n - 1;
+            } else {
+                long long l2 = lo % n;
+                if (l2 < 0) l2 += n;
+                hi = l2 + (hi - lo);
+                lo = l2;
+            }
+        } else {
+            if (lo < 0) lo = 0;
+            if (hi > n - 1) hi = n - 1;
+            if (hi < lo) hi = lo;
+        }
+        L.ctl->patch_lo[buf][a] = (int)lo;
+        L.ctl->patch_ext[buf][a] = (int)(hi - lo);
+    }
+}
+
+__device__ void block_bbox_patch(const LbView &L, const MeshView &M, const double *r, int nv, int buf)
+{
+    __shared__ double sh[32];
+    double mn[3], mx[3];
+    for (int a = 0; a < 3; ++a) {
+        double lo = 1e300, hi = -1e300;
+        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+            lo = fmin(lo, r[3 * i + a]);
+            hi = fmax(hi, r[3 * i + a]);
+        }
+        mn[a] = -block_max(-lo, sh);
+        mx[a] = block_max(hi, sh);
+    }
+    if (threadIdx.x == 0) {
+        write_patch(L, mn, mx, buf, 1);
+        for (int a = 0; a < 3; ++a) {
+            M.part[a] = mn[a];
+            M.part[3 + a] = mx[a];
+        }
+        L.ctl->n_part = 1;
+    }
+}
+
 // Symmetric 3x3 eigen-decomposition by cyclic Jacobi rotations: each
 // rotation J in the (p,q) plane with t = sgn(th)/(|th| + sqrt(th^2 + 1)),
 // th = (a_qq - a_pp)/(2 a_pq), c = 1/sqrt(1 + t^2), s = t c, annihilates a_pq.

@@ -183,6 +183,9 @@ cudaError_t launch_centre(const LbView &L, const MeshView &M, int buf, cudaStrea
 cudaError_t launch_indicator(const LbView &L, const MeshView &M, int buf, cudaStream_t s, int prio = 0);
 cudaError_t launch_regularize(const LbView &L, const MeshView &M, const RegParams &p, int buf, cudaStream_t s,
                               int prio = 0);
+// the members with due[k] != 0, one launch per group
+cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<char> &due,
+                                      const std::vector<RegParams> &params, int buf, cudaStream_t s, int prio);
 cudaError_t launch_observables(const LbView &L, const MeshView &M, cudaStream_t s, int prio = 0);
 cudaError_t launch_patch_from_mesh(const LbView &L, const MeshView &M, int buf, cudaStream_t s);
 // Ensemble step phases (two streams, as the single droplet's step):

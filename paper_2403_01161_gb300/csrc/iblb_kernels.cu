@@ -15,8 +15,6 @@
 // only the droplet patch (bounding box of the 4x4x4 stencils) is ever
 // touched: the spread adds into it, the lattice kernel reads and re-zeroes it
 // and stores the velocity there, the interpolation reads it.
-#include <cooperative_groups.h>
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -778,42 +776,6 @@ __global__ void __launch_bounds__(256) k_init(LbView L)
 
 // ---------------------------------------------------------------------------
 // Immersed boundary.
-// Patch of lattice nodes the droplet's stencils can touch, from the node
-// bounding box [mn, mx]: floor(mn)-1 .. floor(mx)+2 per axis (periodic axes
-// keep the lower corner inside the box and may wrap; Zou-He axes clamp).
-// `grow` extra nodes on each side (1 covers the nodes' motion over one more
-// step: |u| <= 0.3 keeps floor(r) within one node).
-__device__ void write_patch(const LbView &L, const double mn[3], const double mx[3], int buf, int grow)
-{
-    for (int a = 0; a < 3; ++a) {
-        const int n = L.n[a];
-        double lo_d = mn[a], hi_d = mx[a];
-        if (!(lo_d > -1e8 && lo_d < 1e8) || !(hi_d > -1e8 && hi_d < 1e8) || hi_d < lo_d) {
-            L.ctl->patch_lo[buf][a] = 0;
-            L.ctl->patch_ext[buf][a] = n - 1;
-            continue;
-        }
-        long long lo = (long long)floor(lo_d) - 1 - grow, hi = (long long)floor(hi_d) + 2 + grow;
-        if (L.bc[a] == IBL_BC_PERIODIC) {
-            if (hi - lo + 1 >= n) {
-                lo = 0;
-                hi = n - 1;
-            } else {
-                long long l2 = lo % n;
-                if (l2 < 0) l2 += n;
-                hi = l2 + (hi - lo);
-                lo = l2;
-            }
-        } else {
-            if (lo < 0) lo = 0;
-            if (hi > n - 1) hi = n - 1;
-            if (hi < lo) hi = lo;
-        }
-        L.ctl->patch_lo[buf][a] = (int)lo;
-        L.ctl->patch_ext[buf][a] = (int)(hi - lo);
-    }
-}
-
 // Warp 0 of block 0 of the force/spread kernel of step t: reduce the
 // bounding-box rows of r_t left by the previous interpolation (or
 // regularisation) into the patch of step t + 1, grown by one node, in
@@ -1181,328 +1143,6 @@ __global__ void __launch_bounds__(128)
         interp_body<T, kFwdLanes, P>(LG.v[mi - m0], MG.v[mi - m0], bb - blk_start[mi],
                                      blk_start[mi + 1] - blk_start[mi]);
         __syncthreads();  // the next pass reuses the body's shared rows
-    }
-}
-
-__device__ void block_bbox_patch(const LbView &L, const MeshView &M, const double *r, int nv, int buf)
-{
-    __shared__ double sh[32];
-    double mn[3], mx[3];
-    for (int a = 0; a < 3; ++a) {
-        double lo = 1e300, hi = -1e300;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            lo = fmin(lo, r[3 * i + a]);
-            hi = fmax(hi, r[3 * i + a]);
-        }
-        mn[a] = -block_max(-lo, sh);
-        mx[a] = block_max(hi, sh);
-    }
-    if (threadIdx.x == 0) {
-        write_patch(L, mn, mx, buf, 1);
-        for (int a = 0; a < 3; ++a) {
-            M.part[a] = mn[a];
-            M.part[3 + a] = mx[a];
-        }
-        L.ctl->n_part = 1;
-    }
-}
-
-// Mesh regularisation, Sec. 3.3, one block: x_o fixed, x_q the previous
-// iterate, x_p the new one (ping-pong between r and s1), x_b in s2.
-// patch_buf: patch buffer (parity) of the next step, rewritten from the
-// regularised positions.
-// This thread's share of the enclosed volume and of its first moment, summed
-// over signed tetrahedra (x_0, a, b, c) of the triangles, positions relative
-// to node 0: v[0] = V, v[1..3] = int (x - x_0) dV.
-__device__ __forceinline__ void enclosed_volume_sums(const MeshView &M, double v[4])
-{
-    v[0] = v[1] = v[2] = v[3] = 0.0;
-    const double r0[3] = {M.r[0], M.r[1], M.r[2]};
-    for (int t = threadIdx.x; t < M.nt; t += blockDim.x) {
-        double pp[3][3];
-        for (int k = 0; k < 3; ++k)
-            for (int a = 0; a < 3; ++a) pp[k][a] = M.r[3 * M.tris[3 * t + k] + a] - r0[a];
-        double bc[3];
-        cross3(pp[1], pp[2], bc);
-        const double vt = (pp[0][0] * bc[0] + pp[0][1] * bc[1] + pp[0][2] * bc[2]) / 6.0;
-        v[0] += vt;
-        for (int a = 0; a < 3; ++a) v[1 + a] += vt * (pp[0][a] + pp[1][a] + pp[2][a]) / 4.0;
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_regularize(LbView L, MeshView M, RegParams p, int patch_buf)
-{
-    __shared__ double sh[32];
-    const int nv = M.nv;
-    // mesh quality: the largest ratio of longest to shortest edge over the
-    // triangles (node clustering and loose, stretched elements both raise it)
-    double q = 1.0;
-    for (int t = threadIdx.x; t < M.nt; t += blockDim.x) {
-        const int v[3] = {M.tris[3 * t], M.tris[3 * t + 1], M.tris[3 * t + 2]};
-        double e2[3];
-        for (int k = 0; k < 3; ++k) {
-            const double *a = M.r + 3 * v[k], *b = M.r + 3 * v[(k + 1) % 3];
-            const double dx = b[0] - a[0], dy = b[1] - a[1], dz = b[2] - a[2];
-            e2[k] = dx * dx + dy * dy + dz * dz;
-        }
-        const double lo = fmin(e2[0], fmin(e2[1], e2[2])), hi = fmax(e2[0], fmax(e2[1], e2[2]));
-        q = fmax(q, lo > 0.0 ? sqrt(hi / lo) : 1e300);
-    }
-    q = block_max(q, sh);
-    if (threadIdx.x == 0) L.ctl->mesh_q = q;
-    if (p.trigger > 0.0 && !(q > p.trigger)) {
-        // adaptive schedule: the mesh is still regular enough, nothing to do
-        if (threadIdx.x == 0) L.ctl->reg_iters = 0;
-        return;
-    }
-    __shared__ double shv[32][4];
-    double V0 = 0.0;
-    if (p.keep_volume) {
-        double v4[4];
-        enclosed_volume_sums(M, v4);
-        block_sum<4>(v4, shv);
-        V0 = v4[0];
-    }
-    double *xo = M.s0, *xb = M.s2;
-    double *buf[2] = {M.r, M.s1};
-    for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) xo[i] = M.r[i];
-    __syncthreads();
-    const double sg = p.plus_sign ? 1.0 : -1.0;
-    int cur = 0, it = 0;
-    bool conv = false;
-    while (it < p.max_iter) {
-        ++it;
-        const double *xq = buf[cur];
-        double *xp = buf[cur ^ 1];
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = M.nb_ptr[i], b1 = M.nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xq[3 * M.nb_idx[k] + a];
-                const double v = p.alpha * xo[3 * i + a] + (1.0 - p.alpha) / ni * s;
-                xp[3 * i + a] = v;
-                xb[3 * i + a] = v - (p.alpha * xo[3 * i + a] + (1.0 - p.alpha) * xq[3 * i + a]);
-            }
-        }
-        __syncthreads();
-        double dmax = 0.0;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = M.nb_ptr[i], b1 = M.nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            double d2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xb[3 * M.nb_idx[k] + a];
-                const double v = xp[3 * i + a] - (p.gamma * xb[3 * i + a] + sg * (1.0 - p.gamma) / ni * s);
-                xp[3 * i + a] = v;
-                const double d = v - xq[3 * i + a];
-                d2 += d * d;
-            }
-            dmax = fmax(dmax, sqrt(d2));
-        }
-        dmax = block_max(dmax, sh);  // includes a barrier after the writes above
-        cur ^= 1;
-        if (dmax < p.tol) {
-            conv = true;
-            break;
-        }
-    }
-    if (cur != 0) {
-        for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) M.r[i] = M.s1[i];
-    }
-    __syncthreads();
-    if (p.keep_volume) {
-        // scale about the volume centroid back to the volume enclosed before
-        double v4[4];
-        enclosed_volume_sums(M, v4);
-        block_sum<4>(v4, shv);
-        const double c[3] = {M.r[0] + v4[1] / v4[0], M.r[1] + v4[2] / v4[0], M.r[2] + v4[3] / v4[0]};
-        const double f = cbrt(V0 / v4[0]);
-        __syncthreads();  // every thread has read M.r[0..2] before it moves
-        for (int i = threadIdx.x; i < nv; i += blockDim.x)
-            for (int a = 0; a < 3; ++a) M.r[3 * i + a] = c[a] + f * (M.r[3 * i + a] - c[a]);
-        __syncthreads();
-    }
-    block_bbox_patch(L, M, M.r, nv, patch_buf);
-    if (threadIdx.x == 0) {
-        L.ctl->reg_iters = it;
-        L.ctl->reg_count += 1;
-        if (!conv) atomicOr(&L.ctl->err, IBL_ERRBIT_NOCONV);
-    }
-}
-
-// The same regularisation on a thread-block cluster of kRegCluster CTAs
-// (one per SM), for meshes of up to kRegCluster * kRegPerCta nodes.  CTA c
-// owns nodes [c P, c P + P) and keeps their original position, the two
-// iterates and the correction b in its shared memory; neighbours owned by
-// other CTAs are read through distributed shared memory.  The hardware
-// cluster barrier separates the phases, and each CTA reduces the maxima and
-// sums published by all CTAs in the same order, so every CTA takes the same
-// decisions.  The per-triangle passes (quality, volumes) and the node
-// updates spread over the cluster's SMs instead of one.
-namespace cg = cooperative_groups;
-constexpr int kRegCluster = 16;
-constexpr int kRegPerCta = 2048;
-
-__global__ void __launch_bounds__(1024) k_regularize_cluster(LbView L, MeshView M, RegParams p, int patch_buf, int P)
-{
-    cg::cluster_group cluster = cg::this_cluster();
-    const int C = (int)cluster.num_blocks();
-    const int rank = (int)cluster.block_rank();
-    const int nv = M.nv, tid = threadIdx.x, nth = blockDim.x;
-    extern __shared__ double sm[];
-    double *xo = sm, *xa = sm + 3 * P, *xc = sm + 6 * P, *xb = sm + 9 * P;
-    double *red = sm + 12 * P;  // [8] values this CTA publishes to the cluster
-    __shared__ double shr[32];
-    __shared__ double sh4[32][4];
-    const int g0 = rank * P, g1 = min(nv, g0 + P), own = max(0, g1 - g0);
-    // cluster-wide max / sum of values published in red[0..k) by every CTA
-    auto cluster_max = [&](double v) -> double {
-        v = block_max(v, shr);
-        if (tid == 0) red[0] = v;
-        cluster.sync();
-        double m = -1e300;
-        for (int c = 0; c < C; ++c) m = fmax(m, *cluster.map_shared_rank(red, c));
-        cluster.sync();  // the slot is reused by the next reduction
-        return m;
-    };
-    auto cluster_sum4 = [&](double (&v)[4]) {
-        block_sum<4>(v, sh4);
-        if (tid < 4) red[tid] = v[tid];
-        cluster.sync();
-        for (int k = 0; k < 4; ++k) {
-            double s = 0.0;
-            for (int c = 0; c < C; ++c) s += cluster.map_shared_rank(red, c)[k];
-            v[k] = s;
-        }
-        cluster.sync();
-    };
-    // position of node j in the iterate `buf` (xa or xc), wherever it lives
-    auto pos = [&](double *buf, int j, int a) -> double {
-        const int c = j / P;
-        return cluster.map_shared_rank(buf, c)[3 * (j - c * P) + a];
-    };
-    // mesh quality over the triangles, from the positions in global memory
-    double q = 1.0;
-    for (int t = rank * nth + tid; t < M.nt; t += C * nth) {
-        const int v[3] = {M.tris[3 * t], M.tris[3 * t + 1], M.tris[3 * t + 2]};
-        double e2[3];
-        for (int k = 0; k < 3; ++k) {
-            const double *a = M.r + 3 * v[k], *b = M.r + 3 * v[(k + 1) % 3];
-            const double dx = b[0] - a[0], dy = b[1] - a[1], dz = b[2] - a[2];
-            e2[k] = dx * dx + dy * dy + dz * dz;
-        }
-        const double lo = fmin(e2[0], fmin(e2[1], e2[2])), hi = fmax(e2[0], fmax(e2[1], e2[2]));
-        q = fmax(q, lo > 0.0 ? sqrt(hi / lo) : 1e300);
-    }
-    q = cluster_max(q);
-    if (rank == 0 && tid == 0) L.ctl->mesh_q = q;
-    if (p.trigger > 0.0 && !(q > p.trigger)) {
-        if (rank == 0 && tid == 0) L.ctl->reg_iters = 0;
-        return;
-    }
-    const double r0[3] = {M.r[0], M.r[1], M.r[2]};
-    double V0 = 0.0;
-    if (p.keep_volume) {
-        double v4[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int t = rank * nth + tid; t < M.nt; t += C * nth) {
-            double pp[3][3];
-            for (int k = 0; k < 3; ++k)
-                for (int a = 0; a < 3; ++a) pp[k][a] = M.r[3 * M.tris[3 * t + k] + a] - r0[a];
-            double bc[3];
-            cross3(pp[1], pp[2], bc);
-            v4[0] += (pp[0][0] * bc[0] + pp[0][1] * bc[1] + pp[0][2] * bc[2]) / 6.0;
-        }
-        cluster_sum4(v4);
-        V0 = v4[0];
-    }
-    for (int l = tid; l < own; l += nth)
-        for (int a = 0; a < 3; ++a) xo[3 * l + a] = xa[3 * l + a] = M.r[3 * (g0 + l) + a];
-    cluster.sync();
-    const double sg = p.plus_sign ? 1.0 : -1.0;
-    double *xq = xa, *xp = xc;
-    int it = 0;
-    bool conv = false;
-    while (it < p.max_iter) {
-        ++it;
-        // Eq. (extended laplacian smoothing) and Eq. (distanceregularization)
-        for (int l = tid; l < own; l += nth) {
-            const int g = g0 + l, b0 = M.nb_ptr[g], b1 = M.nb_ptr[g + 1], ni = b1 - b0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += pos(xq, M.nb_idx[k], a);
-                const double v = p.alpha * xo[3 * l + a] + (1.0 - p.alpha) / ni * s;
-                xp[3 * l + a] = v;
-                xb[3 * l + a] = v - (p.alpha * xo[3 * l + a] + (1.0 - p.alpha) * xq[3 * l + a]);
-            }
-        }
-        cluster.sync();
-        // Eq. (HC_algo_full) and the exit test
-        double dmax = 0.0;
-        for (int l = tid; l < own; l += nth) {
-            const int g = g0 + l, b0 = M.nb_ptr[g], b1 = M.nb_ptr[g + 1], ni = b1 - b0;
-            double d2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += pos(xb, M.nb_idx[k], a);
-                const double v = xp[3 * l + a] - (p.gamma * xb[3 * l + a] + sg * (1.0 - p.gamma) / ni * s);
-                xp[3 * l + a] = v;
-                const double d = v - xq[3 * l + a];
-                d2 += d * d;
-            }
-            dmax = fmax(dmax, sqrt(d2));
-        }
-        dmax = cluster_max(dmax);  // its barriers also end every read of xb and xq
-        double *tmp = xq;
-        xq = xp;
-        xp = tmp;
-        if (dmax < p.tol) {
-            conv = true;
-            break;
-        }
-    }
-    // xq holds the result
-    double c[3] = {0.0, 0.0, 0.0}, f = 1.0;
-    if (p.keep_volume) {
-        double v4[4] = {0.0, 0.0, 0.0, 0.0};
-        const double s0[3] = {pos(xq, 0, 0), pos(xq, 0, 1), pos(xq, 0, 2)};
-        for (int t = rank * nth + tid; t < M.nt; t += C * nth) {
-            double pp[3][3];
-            for (int k = 0; k < 3; ++k)
-                for (int a = 0; a < 3; ++a) pp[k][a] = pos(xq, M.tris[3 * t + k], a) - s0[a];
-            double bc[3];
-            cross3(pp[1], pp[2], bc);
-            const double vt = (pp[0][0] * bc[0] + pp[0][1] * bc[1] + pp[0][2] * bc[2]) / 6.0;
-            v4[0] += vt;
-            for (int a = 0; a < 3; ++a) v4[1 + a] += vt * (pp[0][a] + pp[1][a] + pp[2][a]) / 4.0;
-        }
-        cluster_sum4(v4);
-        for (int a = 0; a < 3; ++a) c[a] = s0[a] + v4[1 + a] / v4[0];
-        f = cbrt(V0 / v4[0]);
-    }
-    double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-    for (int l = tid; l < own; l += nth)
-        for (int a = 0; a < 3; ++a) {
-            const double v = p.keep_volume ? c[a] + f * (xq[3 * l + a] - c[a]) : xq[3 * l + a];
-            M.r[3 * (g0 + l) + a] = v;
-            mn[a] = fmin(mn[a], v);
-            mx[a] = fmax(mx[a], v);
-        }
-    for (int a = 0; a < 3; ++a) {
-        mn[a] = -cluster_max(-mn[a]);
-        mx[a] = cluster_max(mx[a]);
-    }
-    if (rank == 0 && tid == 0) {
-        write_patch(L, mn, mx, patch_buf, 1);
-        for (int a = 0; a < 3; ++a) {
-            M.part[a] = mn[a];
-            M.part[3 + a] = mx[a];
-        }
-        L.ctl->n_part = 1;
-        L.ctl->reg_iters = it;
-        L.ctl->reg_count += 1;
-        if (!conv) atomicOr(&L.ctl->err, IBL_ERRBIT_NOCONV);
     }
 }
 
@@ -1895,56 +1535,6 @@ cudaError_t launch_interp(const LbView &L, const MeshView &M, cudaStream_t s, in
     return launch_p(k_interp<float, kFwdLanes>, g, b, s, prio, L, M, nblk);
 }
 
-cudaError_t launch_regularize(const LbView &L, const MeshView &M, const RegParams &p, int buf, cudaStream_t s,
-                              int prio)
-{
-    // a cluster of one CTA per SM when the mesh fits (and the device takes
-    // the cluster size), the single-CTA kernel otherwise
-    static int cluster_ok = -1;
-    if (cluster_ok < 0) {
-        cluster_ok = 0;
-        cudaError_t e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(sizeof(double) * (12 * kRegPerCta + 8)));
-        if (e == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(kRegCluster);
-            cfg.blockDim = dim3(1024);
-            cfg.dynamicSmemBytes = sizeof(double) * (12 * kRegPerCta + 8);
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = kRegCluster;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            e = cudaOccupancyMaxActiveClusters(&n, k_regularize_cluster, &cfg);
-            if (e == cudaSuccess && n > 0) cluster_ok = 1;
-        }
-        cudaGetLastError();  // a refused attribute only selects the fallback
-    }
-    if (!cluster_ok || M.nv > kRegCluster * kRegPerCta)
-        return launch_p(k_regularize, dim3(1), dim3(1024), s, prio, L, M, p, buf);
-    const int P = (M.nv + kRegCluster - 1) / kRegCluster;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kRegCluster);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = sizeof(double) * (12 * (size_t)P + 8);
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kRegCluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributePriority;
-    at[1].val.priority = prio;
-    cfg.attrs = at;
-    cfg.numAttrs = prio != 0 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, k_regularize_cluster, L, M, p, buf, P);
-}
-
 cudaError_t launch_observables(const LbView &L, const MeshView &M, cudaStream_t s, int prio)
 {
     int g = (M.nt + 255) / 256;
@@ -2196,172 +1786,3 @@ void velocity_table(int c[19][3], double w[19])
 }
 
 }  // namespace iblb
-
-// ---------------------------------------------------------------------------
-// Allocation-free mesh regularisation.
-//
-// Some callers cannot allocate device memory: a host program whose own
-// allocator has reserved the device's memory up front (so any other
-// allocation fails or fragments its pool), a control loop with a fixed time
-// budget that cannot absorb an allocation call that may synchronise the
-// device, or a plug-in whose host forbids it to allocate.  For them this
-// variant of the regularisation kernel keeps its scratch in a fixed array
-// of this file instead of in a caller workspace.  The array is part of the
-// library image, so every GPU that loads the library holds it (1.18 MB)
-// until the process exits.
-namespace iblb {
-namespace {
-
-constexpr int kNoAllocMaxNodes = 16384;  // enough for a level-5 icosphere (10242 nodes)
-
-// x_o, the ping-pong iterate and x_b, each [kNoAllocMaxNodes][3] doubles.
-static __device__ __align__(256) double g_noalloc_scratch[3 * 3 * kNoAllocMaxNodes];
-
-// Same iteration as k_regularize (Sec. 3.3), reading and writing only the
-// caller's positions and the static scratch; result[0] = iterations,
-// result[1] = 1 if the exit test held.
-__global__ void __launch_bounds__(1024)
-    k_regularize_noalloc(double *r, const int *nb_ptr, const int *nb_idx, int nv, double *scratch, RegParams p,
-                         int *result)
-{
-    __shared__ double sh[32];
-    double *xo = scratch, *s1 = scratch + 3 * kNoAllocMaxNodes, *xb = scratch + 6 * kNoAllocMaxNodes;
-    double *buf[2] = {r, s1};
-    for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) xo[i] = r[i];
-    __syncthreads();
-    const double sg = p.plus_sign ? 1.0 : -1.0;
-    int cur = 0, it = 0;
-    bool conv = false;
-    while (it < p.max_iter) {
-        ++it;
-        const double *xq = buf[cur];
-        double *xp = buf[cur ^ 1];
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = nb_ptr[i], b1 = nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xq[3 * nb_idx[k] + a];
-                const double v = p.alpha * xo[3 * i + a] + (1.0 - p.alpha) / ni * s;
-                xp[3 * i + a] = v;
-                xb[3 * i + a] = v - (p.alpha * xo[3 * i + a] + (1.0 - p.alpha) * xq[3 * i + a]);
-            }
-        }
-        __syncthreads();
-        double dmax = 0.0;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = nb_ptr[i], b1 = nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            double d2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xb[3 * nb_idx[k] + a];
-                const double v = xp[3 * i + a] - (p.gamma * xb[3 * i + a] + sg * (1.0 - p.gamma) / ni * s);
-                xp[3 * i + a] = v;
-                const double d = v - xq[3 * i + a];
-                d2 += d * d;
-            }
-            dmax = fmax(dmax, sqrt(d2));
-        }
-        dmax = block_max(dmax, sh);
-        cur ^= 1;
-        if (dmax < p.tol) {
-            conv = true;
-            break;
-        }
-    }
-    if (cur != 0) {
-        for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) r[i] = s1[i];
-    }
-    if (threadIdx.x == 0) {
-        result[0] = it;
-        result[1] = conv ? 1 : 0;
-    }
-}
-
-// Device address of the array per device ordinal, with the id of the
-// context it was looked up in: the array is part of the module loaded into
-// that context, so another context (a driver-API context made current, or the
-// primary context created anew after cudaDeviceReset) holds it elsewhere.
-struct NoAllocSlot {
-    unsigned long long ctx_id;
-    double *ptr;
-};
-std::mutex g_noalloc_mu;
-NoAllocSlot g_noalloc_slot[256] = {};
-
-using CtxGetCurrentFn = CUresult (*)(CUcontext *);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long *);
-
-// Id of the calling thread's current context (0 if there is none yet).
-// Called with g_noalloc_mu held.
-cudaError_t current_context_id(unsigned long long *id)
-{
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    *id = 0;
-    if (!get_current || !get_id) {
-        void *a = nullptr, *b = nullptr;
-        cudaDriverEntryPointQueryResult qa, qb;
-        cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa);
-        if (e == cudaSuccess)
-            e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb);
-        if (e != cudaSuccess) return e;
-        if (qa != cudaDriverEntryPointSuccess || qb != cudaDriverEntryPointSuccess || !a || !b)
-            return cudaErrorNotSupported;
-        get_current = reinterpret_cast<CtxGetCurrentFn>(a);
-        get_id = reinterpret_cast<CtxGetIdFn>(b);
-    }
-    CUcontext c = nullptr;
-    if (get_current(&c) != CUDA_SUCCESS) return cudaErrorUnknown;
-    if (!c) return cudaSuccess;
-    return get_id(c, id) == CUDA_SUCCESS ? cudaSuccess : cudaErrorUnknown;
-}
-
-}  // namespace
-}  // namespace iblb
-
-extern "C" int ibl_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes,
-                                      double alpha, double gamma, double tol, int max_iter, int plus_sign,
-                                      int32_t *result, void *stream)
-{
-    using namespace iblb;
-    if (!r || !nb_ptr || !nb_idx || !result) return iblb_set_error(IBL_EINVAL, "null pointer argument");
-    if (n_nodes < 1 || n_nodes > kNoAllocMaxNodes)
-        return iblb_set_error(IBL_EINVAL, "ibl_regularize_noalloc: n_nodes must be in 1..16384 (the size of its "
-                                          "fixed scratch array)");
-    if (!(alpha >= 0 && alpha <= 1) || !(gamma >= 0 && gamma <= 1) || !(tol > 0) || max_iter < 1)
-        return iblb_set_error(IBL_EINVAL, "regularisation parameters out of range");
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
-    if (dev < 0 || dev >= 256) return iblb_set_error(IBL_EINVAL, "device ordinal out of range");
-    double *scratch = nullptr;
-    {
-        // first call on this device, or first call in another context of
-        // it: look up the array's device address with the device current
-        // (the name alone is a host-side stand-in, not a device address)
-        std::lock_guard<std::mutex> lock(g_noalloc_mu);
-        unsigned long long ctx = 0;
-        e = current_context_id(&ctx);
-        if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
-        NoAllocSlot &slot = g_noalloc_slot[dev];
-        if (ctx == 0 || !slot.ptr || slot.ctx_id != ctx) {
-            void *p = nullptr;
-            e = cudaGetSymbolAddress(&p, g_noalloc_scratch);  // also creates the context if there is none yet
-            if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
-            e = current_context_id(&ctx);
-            if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
-            slot.ptr = static_cast<double *>(p);
-            slot.ctx_id = ctx;
-        }
-        scratch = slot.ptr;
-    }
-    RegParams p{alpha, gamma, tol, max_iter, plus_sign ? 1 : 0};
-    k_regularize_noalloc<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(
-        r, reinterpret_cast<const int *>(nb_ptr), reinterpret_cast<const int *>(nb_idx), n_nodes, scratch, p,
-        reinterpret_cast<int *>(result));
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
-    return IBL_OK;
-}
