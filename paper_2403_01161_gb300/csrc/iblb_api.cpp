@@ -1185,6 +1185,8 @@ int ibl_lb_create(const ibl_lb_params *p, const double *A_frames, int n_frames, 
     v.omega = 1.0 / p->tau;
     v.omega_f = (float)(1.0 / p->tau);
     v.inv_nx = 1.0f / (float)p->n[0];
+    v.div_nx = iblb::div_by_const(p->n[0]);
+    v.div_nxy = iblb::div_by_const(p->n[0] * p->n[1]);
     v.f = lb->ws + L.f;
     v.force = lb->ws + L.force;
     v.vel = lb->ws + L.vel;

@@ -317,17 +317,27 @@ __device__ __forceinline__ void stencil_weights(const NodeStencil &S, int b, int
     }
 }
 
+// n / d for 0 <= n < 2^31, d >= 2 (see DivBy).
+__device__ __forceinline__ int fast_div(const int n, const DivBy d)
+{
+    return (int)(__umulhi((unsigned)n, d.mul) >> d.shift);
+}
+
 // Whether lattice node (x, y, z) lies in the droplet patch stored in buffer
-// `buf` of control block c (periodic axes wrap).
+// `buf` of control block c (PER: periodic axes wrap).
+template <bool PER = true>
 __device__ __forceinline__ bool node_in_patch(const LbView &L, const Ctl *c, int buf, int x, int y, int z)
 {
-    int dx = x - c->patch_lo[buf][0], dy = y - c->patch_lo[buf][1], dz = z - c->patch_lo[buf][2];
-    if (L.bc[0] == IBL_BC_PERIODIC && dx < 0) dx += L.n[0];
-    if (L.bc[1] == IBL_BC_PERIODIC && dy < 0) dy += L.n[1];
-    if (L.bc[2] == IBL_BC_PERIODIC && dz < 0) dz += L.n[2];
+    // pairs: the rows of patch_lo and patch_ext are 8-byte aligned
+    const int2 lo = *reinterpret_cast<const int2 *>(&c->patch_lo[buf][0]);
+    const int2 ext = *reinterpret_cast<const int2 *>(&c->patch_ext[buf][0]);
+    int dx = x - lo.x, dy = y - lo.y, dz = z - c->patch_lo[buf][2];
+    if (PER && L.bc[0] == IBL_BC_PERIODIC && dx < 0) dx += L.n[0];
+    if (PER && L.bc[1] == IBL_BC_PERIODIC && dy < 0) dy += L.n[1];
+    if (PER && L.bc[2] == IBL_BC_PERIODIC && dz < 0) dz += L.n[2];
     // an empty patch has extent -1: no node is inside
-    return c->patch_ext[buf][0] >= 0 && (unsigned)dx <= (unsigned)c->patch_ext[buf][0] &&
-           (unsigned)dy <= (unsigned)c->patch_ext[buf][1] && (unsigned)dz <= (unsigned)c->patch_ext[buf][2];
+    return ext.x >= 0 && (unsigned)dx <= (unsigned)ext.x && (unsigned)dy <= (unsigned)ext.y &&
+           (unsigned)dz <= (unsigned)c->patch_ext[buf][2];
 }
 
 // Surface-tension force of triangle t on its vertex in position `slot`

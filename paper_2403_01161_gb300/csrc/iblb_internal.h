@@ -33,6 +33,26 @@ struct alignas(128) Ctl {
     int patch_ext[3][4];         // extent (hi - lo), -1 = empty
 };
 
+static_assert(offsetof(Ctl, patch_lo) % 8 == 0 && offsetof(Ctl, patch_ext) % 8 == 0, "patch rows are read in pairs");
+
+// Division of 0 <= n < 2^31 by a fixed d >= 2 as (n mul) >> (32 + shift):
+// with 2^l the power of two at or above d, mul = floor(2^(31 + l) / d) + 1 is
+// below 2^32, and n (mul d - 2^(31 + l)) < 2^31 d <= 2^(31 + l) keeps the
+// quotient exact.
+struct DivBy {
+    unsigned mul;
+    unsigned shift;
+};
+inline DivBy div_by_const(int d)
+{
+    DivBy r;
+    unsigned l = 1;
+    while ((1ll << l) < d) ++l;
+    r.mul = (unsigned)((1ull << (31 + l)) / (unsigned)d + 1);
+    r.shift = l - 1;
+    return r;
+}
+
 // Views handed to kernels by value.
 struct LbView {
     int n[3];
@@ -43,6 +63,7 @@ struct LbView {
     int rule;           // IBL_EDGE_*
     double omega;       // 1 / tau
     float omega_f;
+    DivBy div_nx, div_nxy;  // node -> row and z plane in the single-lattice kernel
     float inv_nx;       // 1 / n[0] (rounded): row of a node within its z plane in the batched lattice kernel
     void *f;            // [19][qs]
     void *force;        // [nodes][4]: x, y, z, 0 (one 16-byte record per node in FP32)

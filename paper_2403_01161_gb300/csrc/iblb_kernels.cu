@@ -190,12 +190,21 @@ __device__ __forceinline__ void bc_dispatch(T (&f)[19], const T (&uw)[3], int ru
 // division is needed.  Indices are 32-bit (19 * stride < 2^31 is checked on
 // the host).  The collision works on opposite pairs (c_i, -c_i), whose
 // equilibrium and source terms share their even parts.
-// Node sets of one lattice launch: every node, reading the droplet patch's
-// force where the node lies in the patch (FULL); only the nodes outside the
-// patch (FAR); only patch nodes (NEAR).  FAR and NEAR launches of the same
-// step may run concurrently: in the AA pattern every population slot is read
-// and written by one node only within a step.
+// Node sets of one lattice launch: every node of a box without a droplet
+// (FULL); only the nodes outside the droplet patch (FAR); only patch nodes
+// (NEAR).  FAR and NEAR launches of the same step may run concurrently: in
+// the AA pattern every population slot is read and written by one node only
+// within a step.  Only patch nodes carry a force, so FULL and FAR compile
+// without the Guo source.
 enum { LAT_FULL = 0, LAT_FAR = 1, LAT_NEAR = 2 };
+
+// Population access: slot i of the node at byte offset `off` of its array.
+// The array's base is the same for all threads, the offset 32 bits.
+template <typename T>
+__device__ __forceinline__ T *slot_at(T *f, const int i, const long long qs, const unsigned off)
+{
+    return reinterpret_cast<T *>(reinterpret_cast<char *>(f + i * qs) + off);
+}
 
 // 3 w_i, the weight of the odd (momentum) parts of the equilibrium and of
 // the Guo source.  The exact values are 1/6 (|c_i|^2 = 1) and 1/12 (|c_i|^2
@@ -214,33 +223,95 @@ __device__ __forceinline__ T odd_weight()
     else return T(3.0 * wgt(i));
 }
 
+// Byte offsets to a node's neighbours along each axis (odd step).  Periodic
+// axes wrap.  On a Zou-He axis a missing neighbour points back at the node
+// itself: a population whose source lies outside the box is an unknown that
+// the boundary rebuild overwrites before anything reads it, so its load only
+// needs an address inside the array, while a store to a missing destination
+// is left out (the flags).
+struct Hops {
+    int xm, xp, ym, yp, zm, zp;
+    bool no_xm, no_xp, no_ym, no_yp, no_zm, no_zp;
+};
+template <typename T, bool PER>
+__device__ __forceinline__ Hops make_hops(const LbView &L, const int x, const int y, const int z)
+{
+    const int nx = L.n[0], ny = L.n[1], nz = L.n[2], S = (int)sizeof(T), Sx = S * nx, Sxy = Sx * ny;
+    const bool px = PER && L.bc[0] == IBL_BC_PERIODIC, py = PER && L.bc[1] == IBL_BC_PERIODIC,
+               pz = PER && L.bc[2] == IBL_BC_PERIODIC;
+    Hops h;
+    h.no_xm = x == 0;
+    h.no_xp = x == nx - 1;
+    h.no_ym = y == 0;
+    h.no_yp = y == ny - 1;
+    h.no_zm = z == 0;
+    h.no_zp = z == nz - 1;
+    h.xm = h.no_xm ? (px ? Sx - S : 0) : -S;
+    h.xp = h.no_xp ? (px ? S - Sx : 0) : S;
+    h.ym = h.no_ym ? (py ? Sxy - Sx : 0) : -Sx;
+    h.yp = h.no_yp ? (py ? Sx - Sxy : 0) : Sx;
+    h.zm = h.no_zm ? (pz ? Sxy * (nz - 1) : 0) : -Sxy;
+    h.zp = h.no_zp ? (pz ? -Sxy * (nz - 1) : 0) : Sxy;
+    if (PER) {
+        h.no_xm = h.no_xm && !px;
+        h.no_xp = h.no_xp && !px;
+        h.no_ym = h.no_ym && !py;
+        h.no_yp = h.no_yp && !py;
+        h.no_zm = h.no_zm && !pz;
+        h.no_zp = h.no_zp && !pz;
+    }
+    return h;
+}
+// Offset of the neighbour along (CX, CY, CZ), and whether it exists.
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ unsigned hop(const Hops &h)
+{
+    unsigned o = 0;
+    if constexpr (CX != 0) o += (unsigned)(CX > 0 ? h.xp : h.xm);
+    if constexpr (CY != 0) o += (unsigned)(CY > 0 ? h.yp : h.ym);
+    if constexpr (CZ != 0) o += (unsigned)(CZ > 0 ? h.zp : h.zm);
+    return o;
+}
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ bool hop_exists(const Hops &h)
+{
+    bool no = false;
+    if constexpr (CX != 0) no = no || (CX > 0 ? h.no_xp : h.no_xm);
+    if constexpr (CY != 0) no = no || (CY > 0 ? h.no_yp : h.no_ym);
+    if constexpr (CZ != 0) no = no || (CZ > 0 ? h.no_zp : h.no_zm);
+    return !no;
+}
+
 // The part of a node update after its 19 incoming populations g are in
 // registers: boundary rebuild (sx, sy, sz: -1 / 0 / +1 where the node lies on
 // a wall of that axis), patch force, moments, BGK + Guo, stores (AA pattern:
 // even step own slots opp(i), odd step slot i at x + c_i), velocity record.
 // Returns whether the node is unstable.
-template <typename T, bool ODD, bool REC, int MODE, bool PER, class P = L2Keep>
+// CEN: the boundary field may be centred on the droplet (L.recentre); false
+// where the host knows it is not, since the offset's FP64 arithmetic would
+// otherwise be issued by every warp with a wall node, predicated off or not
+// (nine FP64 instructions, 16 cycles each per SM).
+template <typename T, bool ODD, bool REC, int MODE, bool PER, bool CEN, class P = L2Keep>
 __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], const int x, const int y, const int z,
-                                               const int node, const bool in_patch, const int pbuf, const int sx,
-                                               const int sy, const int sz)
+                                               const int node, const int pbuf, const int sx, const int sy, const int sz,
+                                               [[maybe_unused]] const Hops &h_)
 {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
-    const int nxy = nx * ny;
+    constexpr bool FORCE = MODE == LAT_NEAR;
     bool bad = false;
     {
         T *__restrict__ f = static_cast<T *>(L.f);
         struct NoKeep {};
         [[maybe_unused]] const std::conditional_t<MODE == LAT_NEAR, P, NoKeep> K;
-        const int qs = (int)L.qs;
-        const bool px = PER && L.bc[0] == IBL_BC_PERIODIC, py = PER && L.bc[1] == IBL_BC_PERIODIC,
-                   pz = PER && L.bc[2] == IBL_BC_PERIODIC;
+        const long long qs = L.qs;
+        [[maybe_unused]] const unsigned noff = (unsigned)node * (unsigned)sizeof(T);
         if (sx | sy | sz) {
             // Eq. (velo_facce_cubo_da_gradiente) in the storage precision,
             // about the box centre or, with re-centring, about the droplet's
             // centre of mass at the start of the step (the offset in FP64)
             const T *A = static_cast<const T *>(L.frames_t) + 9 * L.ctl->frame_par[ODD ? 1 : 0];
             T lx, ly, lz;
-            if (L.recentre) {
+            if (CEN && L.recentre) {
                 const double *c = L.ctl->centre[pbuf];
                 lx = T(double(x) - c[0]);
                 ly = T(double(y) - c[1]);
@@ -258,13 +329,10 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
         // droplet patch: read the spread force (and clear it), store u below;
         // both fields hold a 4-wide record (x, y, z, 0) per node
         T Fx = T(0), Fy = T(0), Fz = T(0);
-        T *__restrict__ force = static_cast<T *>(L.force);
-        if constexpr (MODE == LAT_NEAR) {
+        [[maybe_unused]] T *__restrict__ force = static_cast<T *>(L.force);
+        if constexpr (FORCE) {
             K.ld3(force + 4 * node, Fx, Fy, Fz);
             K.st3(force + 4 * node, T(0), T(0), T(0));
-        } else if (in_patch) {
-            rec_ld3(force + 4 * node, Fx, Fy, Fz);
-            rec_st3(force + 4 * node, T(0), T(0), T(0));
         }
 
         T drho = T(0), jx = T(0), jy = T(0), jz = T(0);
@@ -279,7 +347,12 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
         const T ir = T(1) / rho;
         // rho u = j + F/2 (Eq. (density_velocity_LB)); the odd (momentum)
         // parts of the equilibrium are formed from it directly
-        const T mx = jx + T(0.5) * Fx, my = jy + T(0.5) * Fy, mz = jz + T(0.5) * Fz;
+        T mx = jx, my = jy, mz = jz;
+        if constexpr (FORCE) {
+            mx += T(0.5) * Fx;
+            my += T(0.5) * Fy;
+            mz += T(0.5) * Fz;
+        }
         const T ux = mx * ir, uy = my * ir, uz = mz * ir;
         const T uu = ux * ux + uy * uy + uz * uz;
         bad = !(uu <= T(0.09)) || !(drho == drho);
@@ -292,74 +365,76 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
                 *flag = 0;
             }
         }
-        const T fpre = T(1) - T(0.5) * om;
-        const T uF = ux * Fx + uy * Fy + uz * Fz;
+        [[maybe_unused]] T fpre, uF;
+        if constexpr (FORCE) {
+            fpre = T(1) - T(0.5) * om;
+            uF = ux * Fx + uy * Fy + uz * Fz;
+        }
         const T dmr = drho - rho * (T(1.5) * uu);  // drho - (3/2) rho u.u
         {
             constexpr double w0 = wgt(0);
             const T geq = T(w0) * dmr;
-            const T src = fpre * T(w0) * (T(-3) * uF);
-            g[0] = g[0] + om * (geq - g[0]) + src;
+            g[0] = g[0] + om * (geq - g[0]);
+            if constexpr (FORCE) g[0] += fpre * T(w0) * (T(-3) * uF);
         }
         sfor<9>([&](auto I) {
             constexpr int i = decltype(I)::value + 1;
             constexpr int j = opp(i);
-            T cp = T(0), cF = T(0);  // c_i . rho u, c_i . F
-            if constexpr (cxf(i) != 0) { cp += T(cxf(i)) * mx; cF += T(cxf(i)) * Fx; }
-            if constexpr (cyf(i) != 0) { cp += T(cyf(i)) * my; cF += T(cyf(i)) * Fy; }
-            if constexpr (czf(i) != 0) { cp += T(czf(i)) * mz; cF += T(czf(i)) * Fz; }
+            T cp = T(0);  // c_i . rho u
+            if constexpr (cxf(i) != 0) cp += T(cxf(i)) * mx;
+            if constexpr (cyf(i) != 0) cp += T(cyf(i)) * my;
+            if constexpr (czf(i) != 0) cp += T(czf(i)) * mz;
             const T cu = cp * ir;
             constexpr double w = wgt(i);
             const T w3 = odd_weight<T, i>();
             const T even_eq = T(w) * (T(4.5) * cp * cu + dmr);
             const T odd_eq = w3 * cp;
-            const T even_src = fpre * T(w) * (T(9) * cu * cF - T(3) * uF);
-            const T odd_src = fpre * w3 * cF;
-            g[i] = g[i] + om * (even_eq + odd_eq - g[i]) + (even_src + odd_src);
-            g[j] = g[j] + om * (even_eq - odd_eq - g[j]) + (even_src - odd_src);
+            g[i] = g[i] + om * (even_eq + odd_eq - g[i]);
+            g[j] = g[j] + om * (even_eq - odd_eq - g[j]);
+            if constexpr (FORCE) {
+                T cF = T(0);  // c_i . F
+                if constexpr (cxf(i) != 0) cF += T(cxf(i)) * Fx;
+                if constexpr (cyf(i) != 0) cF += T(cyf(i)) * Fy;
+                if constexpr (czf(i) != 0) cF += T(czf(i)) * Fz;
+                const T even_src = fpre * T(w) * (T(9) * cu * cF - T(3) * uF);
+                const T odd_src = fpre * w3 * cF;
+                g[i] += even_src + odd_src;
+                g[j] += even_src - odd_src;
+            }
         });
 
         if constexpr (!ODD) {
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                if constexpr (MODE == LAT_NEAR) K.st(f + opp(i) * qs + node, g[i]);
-                else f[opp(i) * qs + node] = g[i];
+                if constexpr (MODE == LAT_NEAR) K.st(slot_at(f, opp(i), qs, noff), g[i]);
+                else *slot_at(f, opp(i), qs, noff) = g[i];
             });
         } else {
-            // destination x + c_i, slot i.  The node coordinates pass through
-            // an opaque move, so the neighbour offsets are recomputed here
-            // instead of being held in registers across the collision (which
-            // made this kernel spill).
-            int xs = x, ys = y, zs = z;
-            asm volatile("mov.b32 %0, %0;" : "+r"(xs));
-            asm volatile("mov.b32 %0, %0;" : "+r"(ys));
-            asm volatile("mov.b32 %0, %0;" : "+r"(zs));
-            const int nodes_ = xs + nx * ys + nxy * zs;
-            int sxm = -1, sxp = 1, sym = -nx, syp = nx, szm = -nxy, szp = nxy, smiss = 0;
-            if (xs == 0) { if (px) sxm = nx - 1; else smiss |= 1; }
-            if (xs == nx - 1) { if (px) sxp = -(nx - 1); else smiss |= 2; }
-            if (ys == 0) { if (py) sym = (ny - 1) * nx; else smiss |= 4; }
-            if (ys == ny - 1) { if (py) syp = -(ny - 1) * nx; else smiss |= 8; }
-            if (zs == 0) { if (pz) szm = (nz - 1) * nxy; else smiss |= 16; }
-            if (zs == nz - 1) { if (pz) szp = -(nz - 1) * nxy; else smiss |= 32; }
+            // destination x + c_i, slot i.  The node's own offset passes
+            // through an opaque move, so the neighbour offsets are summed
+            // again here instead of being held in registers across the
+            // collision; the patch-node update, which holds more, forms them
+            // anew from the coordinates (either way the kernel spilled).
+            unsigned here = noff;
+            asm volatile("mov.b32 %0, %0;" : "+r"(here));
+            Hops h = h_;
+            if constexpr (MODE == LAT_NEAR) {
+                int xs = x, ys = y, zs = z;
+                asm volatile("mov.b32 %0, %0;" : "+r"(xs));
+                asm volatile("mov.b32 %0, %0;" : "+r"(ys));
+                asm volatile("mov.b32 %0, %0;" : "+r"(zs));
+                h = make_hops<T, PER>(L, xs, ys, zs);
+            }
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                constexpr int cx = cxf(i), cy = cyf(i), cz = czf(i);
-                constexpr int need = (cx > 0 ? 2 : (cx < 0 ? 1 : 0)) | (cy > 0 ? 8 : (cy < 0 ? 4 : 0)) |
-                                     (cz > 0 ? 32 : (cz < 0 ? 16 : 0));
-                const int off = (cx > 0 ? sxp : (cx < 0 ? sxm : 0)) + (cy > 0 ? syp : (cy < 0 ? sym : 0)) +
-                                (cz > 0 ? szp : (cz < 0 ? szm : 0));
-                if ((smiss & need) == 0) {
-                    if constexpr (MODE == LAT_NEAR) K.st(f + i * qs + nodes_ + off, g[i]);
-                    else f[i * qs + nodes_ + off] = g[i];
+                if (hop_exists<cxf(i), cyf(i), czf(i)>(h)) {
+                    T *a = slot_at(f, i, qs, here + hop<cxf(i), cyf(i), czf(i)>(h));
+                    if constexpr (MODE == LAT_NEAR) K.st(a, g[i]);
+                    else *a = g[i];
                 }
             });
         }
-        if (in_patch) {
-            T *__restrict__ vel = static_cast<T *>(L.vel);
-            if constexpr (MODE == LAT_NEAR) K.st3(vel + 4 * node, ux, uy, uz);
-            else rec_st3(vel + 4 * node, ux, uy, uz);
-        }
+        if constexpr (MODE == LAT_NEAR) K.st3(static_cast<T *>(L.vel) + 4 * node, ux, uy, uz);
         if constexpr (REC) {
             const int nodes = L.nodes;
             T *__restrict__ rec = static_cast<T *>(L.rec);
@@ -379,78 +454,52 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
 // PER: some axis may be periodic (false: every axis has Zou-He walls, so
 // the neighbour offsets are fixed and only the boundary tests remain).
 // P: L2 policy of the patch nodes' accesses (LAT_NEAR).
-template <typename T, bool ODD, bool REC, int MODE, bool PER, class P = L2Keep>
-__device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const int y, const int z, const int pbuf)
+template <typename T, bool ODD, bool REC, int MODE, bool PER, bool CEN, class P = L2Keep>
+__device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const int y, const int z, const int node,
+                                             const int pbuf)
 {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     // the patch of this step lives in buffer pbuf (step % 3)
-    bool in_patch = (MODE == LAT_NEAR);
-    if constexpr (MODE != LAT_NEAR) in_patch = node_in_patch(L, L.ctl, pbuf, x, y, z);
-    if (MODE == LAT_FAR && in_patch) return false;
+    if constexpr (MODE == LAT_FAR) {
+        if (node_in_patch<PER>(L, L.ctl, pbuf, x, y, z)) return false;
+    }
     {
         const int nxy = nx * ny;
-        const int node = x + nx * y + nxy * z;
         T *__restrict__ f = static_cast<T *>(L.f);
         // the patch nodes keep their lines in L2 between steps (see L2Keep)
         struct NoKeep {};
         [[maybe_unused]] const std::conditional_t<MODE == LAT_NEAR, P, NoKeep> K;
-        const int qs = (int)L.qs;
+        const long long qs = L.qs;
         const bool px = PER && L.bc[0] == IBL_BC_PERIODIC, py = PER && L.bc[1] == IBL_BC_PERIODIC,
                    pz = PER && L.bc[2] == IBL_BC_PERIODIC;
         const int sx = px ? 0 : (x == 0 ? -1 : (x == nx - 1 ? 1 : 0));
         const int sy = py ? 0 : (y == 0 ? -1 : (y == ny - 1 ? 1 : 0));
         const int sz = pz ? 0 : (z == 0 ? -1 : (z == nz - 1 ? 1 : 0));
-        // offsets to the neighbours along each axis (odd step: the sources
-        // x - c_i).  Periodic axes wrap.  On a Zou-He axis a missing
-        // neighbour points back at the node itself: a population whose source
-        // lies outside the box is an unknown that the boundary rebuild below
-        // overwrites before anything reads it, so its load only needs an
-        // address inside the array, not a guard.  The patch-node update
-        // (LAT_NEAR) keeps the guard instead (bits of `miss`: 1 x-1, 2 x+1,
-        // 4 y-1, 8 y+1, 16 z-1, 32 z+1), which measured faster there.
-        int oxm = -1, oxp = 1, oym = -nx, oyp = nx, ozm = -nxy, ozp = nxy;
-        [[maybe_unused]] int miss = 0;
-        if constexpr (ODD && MODE == LAT_NEAR) {
-            if (x == 0) { if (px) oxm = nx - 1; else miss |= 1; }
-            if (x == nx - 1) { if (px) oxp = -(nx - 1); else miss |= 2; }
-            if (y == 0) { if (py) oym = (ny - 1) * nx; else miss |= 4; }
-            if (y == ny - 1) { if (py) oyp = -(ny - 1) * nx; else miss |= 8; }
-            if (z == 0) { if (pz) ozm = (nz - 1) * nxy; else miss |= 16; }
-            if (z == nz - 1) { if (pz) ozp = -(nz - 1) * nxy; else miss |= 32; }
-        } else if constexpr (ODD) {
-            if (x == 0) oxm = px ? nx - 1 : 0;
-            if (x == nx - 1) oxp = px ? -(nx - 1) : 0;
-            if (y == 0) oym = py ? (ny - 1) * nx : 0;
-            if (y == ny - 1) oyp = py ? -(ny - 1) * nx : 0;
-            if (z == 0) ozm = pz ? (nz - 1) * nxy : 0;
-            if (z == nz - 1) ozp = pz ? -(nz - 1) * nxy : 0;
-        }
+        // the patch-node update guards its loads too, which measured faster there
+        [[maybe_unused]] Hops h{};
+        if constexpr (ODD) h = make_hops<T, PER>(L, x, y, z);
+        [[maybe_unused]] const unsigned noff = (unsigned)node * (unsigned)sizeof(T);
 
         T g[19];
         if constexpr (!ODD) {
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                if constexpr (MODE == LAT_NEAR) g[i] = K.ld(f + i * qs + node);
-                else g[i] = f[i * qs + node];
+                const T *a = slot_at(f, i, qs, noff);
+                if constexpr (MODE == LAT_NEAR) g[i] = K.ld(a);
+                else g[i] = *a;
             });
         } else {
             // source x - c_i, slot opp(i)
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                constexpr int cx = cxf(i), cy = cyf(i), cz = czf(i);
-                const int off = (cx > 0 ? oxm : (cx < 0 ? oxp : 0)) + (cy > 0 ? oym : (cy < 0 ? oyp : 0)) +
-                                (cz > 0 ? ozm : (cz < 0 ? ozp : 0));
-                if constexpr (MODE == LAT_NEAR) {
-                    constexpr int need = (cx > 0 ? 1 : (cx < 0 ? 2 : 0)) | (cy > 0 ? 4 : (cy < 0 ? 8 : 0)) |
-                                         (cz > 0 ? 16 : (cz < 0 ? 32 : 0));
-                    g[i] = (miss & need) == 0 ? K.ld(f + opp(i) * qs + node + off) : T(0);
-                } else {
-                    g[i] = f[opp(i) * qs + node + off];
-                }
+                const T *a = slot_at(f, opp(i), qs, noff + hop<-cxf(i), -cyf(i), -czf(i)>(h));
+                if constexpr (MODE == LAT_NEAR)
+                    g[i] = hop_exists<-cxf(i), -cyf(i), -czf(i)>(h) ? K.ld(a) : T(0);
+                else g[i] = *a;
             });
         }
 
-        return lattice_finish<T, ODD, REC, MODE, PER, P>(L, g, x, y, z, node, in_patch, pbuf, sx, sy, sz);
+        return lattice_finish<T, ODD, REC, MODE, PER, CEN, P>(L, g, x, y, z, node, pbuf, sx, sy, sz, h);
     }
 }
 
@@ -468,27 +517,36 @@ __device__ __forceinline__ void close_step(const LbView &L)
     L.ctl->frame_par[s & 1] = (int)(k < L.n_frames - 1 ? k : L.n_frames - 1);
 }
 
-template <typename T, bool ODD, bool REC, int MODE, bool PER>
+// One node per thread, 128 consecutive nodes of the flattened box per block,
+// so that every lane works in a box of any size (rows of 200 nodes left 22% of
+// the lanes of row-aligned blocks idle) and every warp's run starts on a
+// 128-byte line of each population array.  Co-limited by HBM and instruction
+// issue: without the force terms where there is no force, and with 32-bit
+// offsets on common bases, a 64^3 far launch issues 536 (even) / 730 (odd)
+// instructions per warp against 643 / 765 before.  Per step: 97 x 75 x 61
+// channel 16.5 -> 12.3 us, 200^3 regularised 228 -> 212 us, 128^3 droplet
+// 57.1 -> 55.0 us, 256^3 within 0.3%.
+template <typename T, bool ODD, bool REC, int MODE, bool PER, bool CEN>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 4) k_lattice(LbView L, int pbuf, int ahead)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x | threadIdx.y) == 0) close_step(L);
-    // L2 prefetch of this thread's node `ahead` z-planes on, which a block of
-    // about one resident wave later updates: its loads then find the lines in
-    // L2 instead of waiting on DRAM behind the stream (ahead = 0: none; the
-    // host leaves it out for a large droplet patch, see L.prefetch)
-    const int za = z + ahead;
-    if (ahead > 0 && za < L.n[2] && x < L.n[0] && y < L.n[1]) {
-        const T *f = static_cast<const T *>(L.f);
-        const int na = x + L.n[0] * (y + L.n[1] * za);
-        const int qs = (int)L.qs;
+    const int node = (int)(blockIdx.x * 128u + threadIdx.x);
+    if (node == 0) close_step(L);
+    // L2 prefetch of the node `ahead` nodes on, which a block of about one
+    // resident wave later updates: its loads then find the lines in L2
+    // instead of waiting on DRAM behind the stream (ahead = 0: none; the host
+    // leaves it out for a large droplet patch, see L.prefetch)
+    if (ahead > 0 && node + ahead < L.nodes) {
+        T *f = static_cast<T *>(L.f);
+        const unsigned off = (unsigned)(node + ahead) * (unsigned)sizeof(T);
 #pragma unroll
-        for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(f + i * qs + na));
+        for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(slot_at(f, i, L.qs, off)));
     }
     bool bad = false;
-    if (x < L.n[0] && y < L.n[1]) bad = lattice_node<T, ODD, REC, MODE, PER>(L, x, y, z, pbuf);
+    if (node < L.nodes) {
+        const int z = fast_div(node, L.div_nxy), p = node - z * L.n[0] * L.n[1];
+        const int y = fast_div(p, L.div_nx), x = p - y * L.n[0];
+        bad = lattice_node<T, ODD, REC, MODE, PER, CEN>(L, x, y, z, node, pbuf);
+    }
     // sticky instability flag, one atomic per warp at most
     const unsigned m = __ballot_sync(0xffffffffu, bad);
     if (m != 0u && (threadIdx.x & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
@@ -633,8 +691,7 @@ __global__ void __launch_bounds__(NT, (B > 768 / NT ? B : 768 / NT)) k_lattice_s
         bool bad = false;
         if (n < nodes) {
             const int z = div_by(n, nxy, inv_nxy), rem = n - z * nxy, y = div_by(rem, nx, inv_nx), x = rem - y * nx;
-            const bool in_patch = node_in_patch(L, L.ctl, pbuf, x, y, z);
-            if (!(MODE == LAT_FAR && in_patch)) {
+            if (MODE != LAT_FAR || !node_in_patch<false>(L, L.ctl, pbuf, x, y, z)) {
                 const int sx = x == 0 ? -1 : (x == nx - 1 ? 1 : 0);
                 const int sy = y == 0 ? -1 : (y == ny - 1 ? 1 : 0);
                 const int sz = z == 0 ? -1 : (z == nz - 1 ? 1 : 0);
@@ -645,7 +702,9 @@ __global__ void __launch_bounds__(NT, (B > 768 / NT ? B : 768 / NT)) k_lattice_s
                     if constexpr (ODD) g[i] = src[i * RUN + (int)((dpack >> (2 * i)) & 3u)];
                     else g[i] = src[i * RUN];
                 });
-                bad = lattice_finish<float, ODD, false, MODE, false>(L, g, x, y, z, n, in_patch, pbuf, sx, sy, sz);
+                Hops h{};
+                if constexpr (ODD) h = make_hops<float, false>(L, x, y, z);
+                bad = lattice_finish<float, ODD, false, MODE, false, true>(L, g, x, y, z, n, pbuf, sx, sy, sz, h);
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, bad);
@@ -679,7 +738,7 @@ __device__ __forceinline__ void patch_rows(const LbView &L, const int buf, const
             if (x0 + lane < ex) {
                 int x = lx + x0 + lane;
                 if (x >= L.n[0]) x -= L.n[0];
-                bad = lattice_node<T, ODD, REC, LAT_NEAR, PER, P>(L, x, y, z, buf);
+                bad = lattice_node<T, ODD, REC, LAT_NEAR, PER, true, P>(L, x, y, z, x + L.n[0] * (y + L.n[1] * z), buf);
             }
             const unsigned m = __ballot_sync(0xffffffffu, bad);
             if (m != 0u && lane == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
@@ -707,7 +766,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lattice_near(Lb
 // that member's step, as the single-droplet far kernel does.  Each thread
 // prefetches into L2 its (x, y) `ahead` planes further (about `waves`
 // resident waves of blocks later).
-template <typename T, bool ODD, int NT, bool PER>
+template <typename T, bool ODD, int NT, bool PER, bool CEN>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT)
     k_lattice_batched(const __grid_constant__ LbGroup G, const int m0, const int b0,
                       const int *__restrict__ blk_member, const int *__restrict__ blk_start, const int pbuf,
@@ -724,17 +783,16 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT)
     if (ahead_nodes > 0) {
         const int za = z + (ahead_nodes + nxy - 1) / nxy;
         if (za < L.n[2] && p < nxy) {
-            const T *f = static_cast<const T *>(L.f);
-            const int na = p + nxy * za;
-            const int qs = (int)L.qs;
+            T *f = static_cast<T *>(L.f);
+            const unsigned off = (unsigned)(p + nxy * za) * (unsigned)sizeof(T);
 #pragma unroll
-            for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(f + i * qs + na));
+            for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(slot_at(f, i, L.qs, off)));
         }
     }
     bool bad = false;
     if (p < nxy) {
         const int y = (int)(((float)p + 0.5f) * L.inv_nx);
-        bad = lattice_node<T, ODD, false, LAT_FAR, PER>(L, p - y * nx, y, z, pbuf);
+        bad = lattice_node<T, ODD, false, LAT_FAR, PER, CEN>(L, p - y * nx, y, z, p + z * nxy, pbuf);
     }
     const unsigned m = __ballot_sync(0xffffffffu, bad);
     if (m != 0u && (threadIdx.x & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
@@ -1307,35 +1365,35 @@ cudaError_t launch_init(const LbView &L, cudaStream_t s)
     return cudaGetLastError();
 }
 
-static void lattice_grid(const LbView &L, dim3 &grid, dim3 &block)
-{
-    // 128-thread blocks (8 per SM at 64 registers): a concurrently running
-    // droplet-kernel block then displaces an eighth of an SM's lattice work
-    // rather than a quarter
-    const int bx = L.n[0] >= 128 ? 128 : ((L.n[0] + 31) / 32) * 32;
-    const int by = 128 / bx;
-    block = dim3(bx, by, 1);
-    grid = dim3((L.n[0] + bx - 1) / bx, (L.n[1] + by - 1) / by, L.n[2]);
-}
-
 static bool any_periodic(const LbView &L)
 {
     return L.bc[0] == IBL_BC_PERIODIC || L.bc[1] == IBL_BC_PERIODIC || L.bc[2] == IBL_BC_PERIODIC;
 }
 
-template <typename T, bool ODD, bool REC>
-static void lattice_launch_t(const LbView &L, int mode, int pbuf, dim3 g, dim3 b, cudaStream_t s)
+// Variants: a recording launch takes the general (periodic) form, and CEN
+// (re-centring) exists only where a droplet does.
+template <typename T, bool ODD>
+static void lattice_launch_t(const LbView &L, bool rec, int mode, int pbuf, cudaStream_t s)
 {
-    // prefetch distance: the z-planes one wave of resident blocks covers
-    const long long wave = (long long)sm_count() * (sizeof(T) == 4 ? 8 : 4), plane = (long long)g.x * g.y;
-    const int ahead = L.prefetch ? (int)((wave + plane - 1) / plane) : 0;
-    if (any_periodic(L)) {
-        if (mode == LAT_FAR) k_lattice<T, ODD, REC, LAT_FAR, true><<<g, b, 0, s>>>(L, pbuf, ahead);
-        else k_lattice<T, ODD, REC, LAT_FULL, true><<<g, b, 0, s>>>(L, pbuf, ahead);
+    const unsigned g = blocks_for(L.nodes, 128);
+    // prefetch distance: the nodes one wave of resident blocks covers
+    const int ahead = L.prefetch ? sm_count() * (sizeof(T) == 4 ? 8 : 4) * 128 : 0;
+    const bool per = any_periodic(L), cen = L.recentre != 0;
+#define IBL_LAUNCH(R, M, P, C) k_lattice<T, ODD, R, M, P, C><<<g, 128, 0, s>>>(L, pbuf, ahead)
+    if (mode != LAT_FAR) {
+        if (rec) IBL_LAUNCH(true, LAT_FULL, true, false);
+        else if (per) IBL_LAUNCH(false, LAT_FULL, true, false);
+        else IBL_LAUNCH(false, LAT_FULL, false, false);
+    } else if (cen) {
+        if (rec) IBL_LAUNCH(true, LAT_FAR, true, true);
+        else if (per) IBL_LAUNCH(false, LAT_FAR, true, true);
+        else IBL_LAUNCH(false, LAT_FAR, false, true);
     } else {
-        if (mode == LAT_FAR) k_lattice<T, ODD, REC, LAT_FAR, false><<<g, b, 0, s>>>(L, pbuf, ahead);
-        else k_lattice<T, ODD, REC, LAT_FULL, false><<<g, b, 0, s>>>(L, pbuf, ahead);
+        if (rec) IBL_LAUNCH(true, LAT_FAR, true, false);
+        else if (per) IBL_LAUNCH(false, LAT_FAR, true, false);
+        else IBL_LAUNCH(false, LAT_FAR, false, false);
     }
+#undef IBL_LAUNCH
 }
 
 // Opts a kernel into its dynamic shared memory and the largest shared-memory
@@ -1424,24 +1482,12 @@ cudaError_t launch_lattice(const LbView &L, bool odd, bool record, int mode, int
 {
     if (L.staged > 0 && !record && staged_ok(L))
         return odd ? staged_dispatch<true>(L, mode, pbuf, s) : staged_dispatch<false>(L, mode, pbuf, s);
-    dim3 g, b;
-    lattice_grid(L, g, b);
     if (L.precision == IBL_FP64) {
-        if (odd) {
-            if (record) lattice_launch_t<double, true, true>(L, mode, pbuf, g, b, s);
-            else lattice_launch_t<double, true, false>(L, mode, pbuf, g, b, s);
-        } else {
-            if (record) lattice_launch_t<double, false, true>(L, mode, pbuf, g, b, s);
-            else lattice_launch_t<double, false, false>(L, mode, pbuf, g, b, s);
-        }
+        if (odd) lattice_launch_t<double, true>(L, record, mode, pbuf, s);
+        else lattice_launch_t<double, false>(L, record, mode, pbuf, s);
     } else {
-        if (odd) {
-            if (record) lattice_launch_t<float, true, true>(L, mode, pbuf, g, b, s);
-            else lattice_launch_t<float, true, false>(L, mode, pbuf, g, b, s);
-        } else {
-            if (record) lattice_launch_t<float, false, true>(L, mode, pbuf, g, b, s);
-            else lattice_launch_t<float, false, false>(L, mode, pbuf, g, b, s);
-        }
+        if (odd) lattice_launch_t<float, true>(L, record, mode, pbuf, s);
+        else lattice_launch_t<float, false>(L, record, mode, pbuf, s);
     }
     return cudaGetLastError();
 }
@@ -1675,7 +1721,7 @@ cudaError_t launch_ensemble_near(const EnsembleView &E, long long step, cudaStre
     return cudaSuccess;
 }
 
-template <typename T, bool ODD, bool PER>
+template <typename T, bool ODD, bool PER, bool CEN>
 static void far_batched_t(const EnsembleView &E, int m0, int pbuf, int waves, int ti, cudaStream_t s)
 {
     const int m1 = m0 + kGroup < (int)E.lv.size() ? m0 + kGroup : (int)E.lv.size();
@@ -1685,9 +1731,25 @@ static void far_batched_t(const EnsembleView &E, int m0, int pbuf, int waves, in
     const int ahead = waves * sm_count() * per_sm * nt;
     Groups &G = groups();
     if (nt == 128)
-        k_lattice_batched<T, ODD, 128, PER><<<lbn, 128, 0, s>>>(G.lg, m0, lb0, E.lat_member[ti], E.lat_start_d[ti], pbuf, ahead);
+        k_lattice_batched<T, ODD, 128, PER, CEN><<<lbn, 128, 0, s>>>(G.lg, m0, lb0, E.lat_member[ti], E.lat_start_d[ti], pbuf, ahead);
     else
-        k_lattice_batched<T, ODD, 256, PER><<<lbn, 256, 0, s>>>(G.lg, m0, lb0, E.lat_member[ti], E.lat_start_d[ti], pbuf, ahead);
+        k_lattice_batched<T, ODD, 256, PER, CEN><<<lbn, 256, 0, s>>>(G.lg, m0, lb0, E.lat_member[ti], E.lat_start_d[ti], pbuf, ahead);
+}
+
+template <typename T>
+static void far_batched_p(const EnsembleView &E, bool odd, bool per, bool cen, int m0, int pbuf, int waves, int ti,
+                          cudaStream_t s)
+{
+#define IBL_LAUNCH(P, C)                                                   \
+    do {                                                                   \
+        if (odd) far_batched_t<T, true, P, C>(E, m0, pbuf, waves, ti, s);  \
+        else far_batched_t<T, false, P, C>(E, m0, pbuf, waves, ti, s);     \
+    } while (0)
+    if (per && cen) IBL_LAUNCH(true, true);
+    else if (per) IBL_LAUNCH(true, false);
+    else if (cen) IBL_LAUNCH(false, true);
+    else IBL_LAUNCH(false, false);
+#undef IBL_LAUNCH
 }
 
 cudaError_t launch_ensemble_far(const EnsembleView &E, long long step, cudaStream_t s)
@@ -1700,25 +1762,13 @@ cudaError_t launch_ensemble_far(const EnsembleView &E, long long step, cudaStrea
     for (int m0 = 0; m0 < n; m0 += kGroup) {
         const int m1 = m0 + kGroup < n ? m0 + kGroup : n;
         fill_group(E, m0, m1);
-        bool per = false;
-        for (int k = m0; k < m1; ++k) per = per || any_periodic(E.lv[k]);
-        if (E.precision == IBL_FP64) {
-            if (per) {
-                if (odd) far_batched_t<double, true, true>(E, m0, pbuf, waves, ti, s);
-                else far_batched_t<double, false, true>(E, m0, pbuf, waves, ti, s);
-            } else {
-                if (odd) far_batched_t<double, true, false>(E, m0, pbuf, waves, ti, s);
-                else far_batched_t<double, false, false>(E, m0, pbuf, waves, ti, s);
-            }
-        } else {
-            if (per) {
-                if (odd) far_batched_t<float, true, true>(E, m0, pbuf, waves, ti, s);
-                else far_batched_t<float, false, true>(E, m0, pbuf, waves, ti, s);
-            } else {
-                if (odd) far_batched_t<float, true, false>(E, m0, pbuf, waves, ti, s);
-                else far_batched_t<float, false, false>(E, m0, pbuf, waves, ti, s);
-            }
+        bool per = false, cen = false;
+        for (int k = m0; k < m1; ++k) {
+            per = per || any_periodic(E.lv[k]);
+            cen = cen || E.lv[k].recentre != 0;
         }
+        if (E.precision == IBL_FP64) far_batched_p<double>(E, odd, per, cen, m0, pbuf, waves, ti, s);
+        else far_batched_p<float>(E, odd, per, cen, m0, pbuf, waves, ti, s);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
