@@ -32,39 +32,19 @@
 namespace iblb {
 namespace {
 
-// phi'(x) of the Peskin 4-point stencil (derivative of Sec. 3.1's phi).
+// Weights of the lane's x-row and of its y and z rows, with derivatives.
 template <typename T>
-__device__ __forceinline__ T peskin_dphi(T x)
-{
-    const T a = fabs(x);
-    const T sg = x < T(0) ? T(-1) : T(1);
-    if (a < T(1)) return sg * T(0.125) * (T(-2) + (T(2) - T(4) * a) / sqrt(T(1) + T(4) * a - T(4) * a * a));
-    if (a < T(2)) return sg * T(0.125) * (T(-2) - (T(6) - T(4) * a) / sqrt(T(-7) + T(12) * a - T(4) * a * a));
-    return T(0);
-}
-
-template <typename T>
-__device__ __forceinline__ void stencil_weights_d(const NodeStencil &S, int b, int c, T w[4], T dw[4], T &wy, T &dwy,
+__device__ __forceinline__ void stencil_weights_d(const NodeStencil<T> &S, int b, int c, T w[4], T dw[4], T &wy, T &dwy,
                                                   T &wz, T &dwz)
 {
-    T fx, fy, fz;
-    if constexpr (sizeof(T) == 8) {
-        fx = S.frac[0];
-        fy = S.frac[1];
-        fz = S.frac[2];
-    } else {
-        fx = T(S.frac[0]);
-        fy = T(S.frac[1]);
-        fz = T(S.frac[2]);
-    }
     for (int a = 0; a < 4; ++a) {
-        w[a] = peskin_phi<T>(fx + T(1 - a));
-        dw[a] = peskin_dphi<T>(fx + T(1 - a));
+        w[a] = stencil_w(S.f[0], S.s[0], a);
+        dw[a] = stencil_dw(S.ds[0], a);
     }
-    wy = peskin_phi<T>(fy + T(1 - b));
-    dwy = peskin_dphi<T>(fy + T(1 - b));
-    wz = peskin_phi<T>(fz + T(1 - c));
-    dwz = peskin_dphi<T>(fz + T(1 - c));
+    wy = stencil_w(S.f[1], S.s[1], b);
+    dwy = stencil_dw(S.ds[1], b);
+    wz = stencil_w(S.f[2], S.s[2], c);
+    dwz = stencil_dw(S.ds[2], c);
 }
 
 // Transpose of a buried link's moving-wall share 3 w_j (c_j.u_w).
@@ -454,21 +434,20 @@ __global__ void __launch_bounds__(128) k_adj_interp(LbView L, MeshView M, AdjVie
     const int lane = threadIdx.x % kLanesPerNode;
     const bool valid = gid < M.nv;
     const int i = valid ? gid : M.nv - 1;
-    const NodeStencil S = node_stencil(L, M.r + 3 * i, lane);
+    double ra;
+    const NodeStencil<T> S = node_stencil<T, kLanesPerNode, true>(L, M.r + 3 * i, lane, L2Plain(), ra);
     const double lr[3] = {J.lam_r[3 * i], J.lam_r[3 * i + 1], J.lam_r[3 * i + 2]};
     T g[3] = {T(0), T(0), T(0)};
     if (valid && S.ok) {
-        const bool perx = L.bc[0] == IBL_BC_PERIODIC, pery = L.bc[1] == IBL_BC_PERIODIC,
-                   perz = L.bc[2] == IBL_BC_PERIODIC;
         const int b = lane & 3, c = lane >> 2;
         T w[4], dw[4], wy, dwy, wz, dwz;
         stencil_weights_d<T>(S, b, c, w, dw, wy, dwy, wz, dwz);
         const int nx = L.n[0], nxy = L.n[0] * L.n[1], nodes = L.nodes;
-        const int row = wrap_index(S.base[1] + b, L.n[1], pery) * nx + wrap_index(S.base[2] + c, L.n[2], perz) * nxy;
+        const int row = stencil_at(S.base[1], b, L.n[1]) * nx + stencil_at(S.base[2], c, L.n[2]) * nxy;
         T *lu = static_cast<T *>(J.lam_u);  // [nodes][4]
         const T lrx = T(lr[0]), lry = T(lr[1]), lrz = T(lr[2]);
         for (int a = 0; a < 4; ++a) {
-            const int id = row + wrap_index(S.base[0] + a, nx, perx);
+            const int id = row + stencil_at(S.base[0], a, nx);
             const T dl = w[a] * wy * wz;
             rec_red3(lu + 4 * id, lrx * dl, lry * dl, lrz * dl);
             const T ul = rec[nodes + id] * lrx + rec[2 * nodes + id] * lry + rec[3 * nodes + id] * lrz;
@@ -505,9 +484,7 @@ __global__ void __launch_bounds__(128) k_adj_surface(LbView L, MeshView M, AdjVi
     #pragma unroll
     for (int k = 0; k < 3; ++k) vid[k] = M.tris[3 * t + k];
     T lk[3][3], Gk[3][3][3];
-    const bool perx = L.bc[0] == IBL_BC_PERIODIC, pery = L.bc[1] == IBL_BC_PERIODIC,
-               perz = L.bc[2] == IBL_BC_PERIODIC;
-    const int nx = L.n[0], nxy = L.n[0] * L.n[1], nodes = L.nodes;
+    const int nx = L.n[0], nxy = L.n[0] * L.n[1];
     const T *lF = static_cast<const T *>(J.lam_F);
     #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -517,16 +494,17 @@ __global__ void __launch_bounds__(128) k_adj_surface(LbView L, MeshView M, AdjVi
             #pragma unroll
             for (int b = 0; b < 3; ++b) Gk[k][c][b] = T(0);
         }
-        const NodeStencil S = node_stencil(L, M.r + 3 * vid[k], lane);
+        double ra;
+        const NodeStencil<T> S = node_stencil<T, kLanesPerNode, true>(L, M.r + 3 * vid[k], lane, L2Plain(), ra);
         if (valid && S.ok) {
             const int b = lane & 3, c = lane >> 2;
             T w[4], dw[4], wy, dwy, wz, dwz;
             stencil_weights_d<T>(S, b, c, w, dw, wy, dwy, wz, dwz);
             const int row =
-                wrap_index(S.base[1] + b, L.n[1], pery) * nx + wrap_index(S.base[2] + c, L.n[2], perz) * nxy;
+                stencil_at(S.base[1], b, L.n[1]) * nx + stencil_at(S.base[2], c, L.n[2]) * nxy;
 #pragma unroll
             for (int a4 = 0; a4 < 4; ++a4) {
-                const int id = row + wrap_index(S.base[0] + a4, nx, perx);
+                const int id = row + stencil_at(S.base[0], a4, nx);
                 T f[3];
                 rec_ld3(lF + 4 * id, f[0], f[1], f[2]);
                 const T wt = w[a4] * wy * wz;

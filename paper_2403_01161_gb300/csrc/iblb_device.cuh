@@ -59,16 +59,6 @@ __host__ __device__ constexpr bool unknown_dir(int j)
     return (SX != 0 && cxf(j) * SX < 0) || (SY != 0 && cyf(j) * SY < 0) || (SZ != 0 && czf(j) * SZ < 0);
 }
 
-// Peskin 4-point stencil phi (Sec. 3.1), in the storage precision T.
-template <typename T>
-__device__ __forceinline__ T peskin_phi(T x)
-{
-    const T a = fabs(x);
-    if (a < T(1)) return T(0.125) * (T(3) - T(2) * a + sqrt(T(1) + T(4) * a - T(4) * a * a));
-    if (a < T(2)) return T(0.125) * (T(5) - T(2) * a - sqrt(T(-7) + T(12) * a - T(4) * a * a));
-    return T(0);
-}
-
 template <typename V>
 __device__ __forceinline__ void cross3(const V a[3], const V b[3], V o[3])
 {
@@ -77,37 +67,10 @@ __device__ __forceinline__ void cross3(const V a[3], const V b[3], V o[3])
     o[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// The 4-point stencil along one axis starts at base = floor(r) - 1.  On a
-// Zou-He axis all four nodes must be interior (1..n-2); periodic axes wrap.
-struct AxisStencil {
-    int base;
-    bool ok;
-};
-__device__ __forceinline__ AxisStencil axis_stencil(double ra, int n, bool periodic)
-{
-    AxisStencil A;
-    A.ok = fabs(ra) < 1e8;
-    A.base = A.ok ? (int)floor(ra) - 1 : 0;
-    if (A.ok && !periodic) A.ok = A.base >= 1 && A.base + 3 <= n - 2;
-    return A;
-}
-__device__ __forceinline__ int wrap_index(int g, int n, bool periodic)
-{
-    if (periodic) {
-        g %= n;
-        if (g < 0) g += n;
-    }
-    return g;
-}
-
 constexpr int kLanesPerNode = 16;  // lane = (b, c) row of the 4x4x4 stencil
 constexpr int kIbThreads = 128;    // threads per block of the node-group kernels
 static_assert(kFwdNodesPerBlock * kFwdLanes == kIbThreads, "forward node-group blocks");
 
-// Per-node stencil of the 16-lane group: lanes 0..2 compute, in FP64, the
-// origin base_a = floor(r_a) - 1 and the exact fraction r_a - floor(r_a) of
-// axis a, and every lane receives all three by shuffles.  The offset of
-// stencil point k is then frac + (1 - k), the correctly rounded r - (base+k).
 // L2 residency of the droplet-side working set.  Every step the outside
 // lattice update streams the whole population array (about twice the L2 of
 // a 128^3 box) through L2, which would evict the mesh arrays, the patch's
@@ -261,60 +224,90 @@ struct L2Plain {
     }
 };
 
+// Population access: slot i of the node at byte offset `off` of its array.
+// The array's base is the same for all threads, the offset 32 bits.
+template <typename T>
+__device__ __forceinline__ T *slot_at(T *f, const int i, const long long qs, const unsigned off)
+{
+    return reinterpret_cast<T *>(reinterpret_cast<char *>(f + i * qs) + off);
+}
+
+// Peskin 4-point stencil of a mesh node (Sec. 3.1).  Along an axis it covers
+// the lattice points base .. base + 3, base = floor(r) - 1; on a Zou-He axis
+// all four must be interior (1..n-2), periodic axes wrap.  With f = r -
+// floor(r) the four values of phi share one square root, s = sqrt(1 + 4 f (1
+// - f)):
+//   phi(f+1), phi(f), phi(f-1), phi(f-2)
+//     = (3 - 2f - s)/8, (3 - 2f + s)/8, (1 + 2f + s)/8, (1 + 2f - s)/8,
+// and their derivatives in r s' = (2 - 4f)/s.  Lanes 0..2 of a node's group
+// evaluate their axis (floor and f in FP64, the rest in the storage type) and
+// every lane receives all three by shuffles: one root per node and axis
+// instead of two branches with a root each for every weight of every lane.
+template <typename T>
 struct NodeStencil {
-    int base[3];
-    double frac[3];
+    int base[3];  // wrapped into the box
+    T f[3], s[3], ds[3];  // ds only with DERIV
     bool ok;
 };
-template <int LANES = kLanesPerNode, class P = L2Keep>
-__device__ __forceinline__ NodeStencil node_stencil(const LbView &L, const double *r, int lane,
-                                                    const P *keep = nullptr)
+// `ra` receives the lane's coordinate (lanes 0..2).
+template <typename T, int LANES, bool DERIV, class P>
+__device__ __forceinline__ NodeStencil<T> node_stencil(const LbView &L, const double *r, int lane, const P &K, double &ra)
 {
-    double ra = 0.0, fr = 0.0;
-    int base = 0;
-    bool ok = true;
+    constexpr int kNone = -2147483647 - 1;
+    int base = kNone;
+    T f = T(0), s = T(1), ds = T(0);
+    ra = 0.0;
     if (lane < 3) {
-        ra = keep ? keep->ld(r + lane) : r[lane];
+        ra = K.ld(r + lane);
         // select by value: indexing the parameter arrays with a runtime lane
         // would copy the kernel parameters to local memory
-        const int na = lane == 0 ? L.n[0] : (lane == 1 ? L.n[1] : L.n[2]);
-        const int bca = lane == 0 ? L.bc[0] : (lane == 1 ? L.bc[1] : L.bc[2]);
-        const AxisStencil A = axis_stencil(ra, na, bca == IBL_BC_PERIODIC);
-        ok = A.ok;
-        base = A.base;
-        fr = ok ? ra - floor(ra) : 0.0;
+        const int n = lane == 0 ? L.n[0] : (lane == 1 ? L.n[1] : L.n[2]);
+        const bool per = (lane == 0 ? L.bc[0] : (lane == 1 ? L.bc[1] : L.bc[2])) == IBL_BC_PERIODIC;
+        // |ra| < 1e8, from the exponent and leading bits (false for NaN)
+        const bool finite = (__double2hiint(ra) & 0x7fffffff) < 0x4197D784;
+        const int fl = finite ? __double2int_rd(ra) : 0;
+        f = T(finite ? ra - (double)fl : 0.0);
+        s = sqrt(fma(T(4) * f, T(1) - f, T(1)));
+        if constexpr (DERIV) ds = (T(2) - T(4) * f) / s;
+        int b = fl - 1;
+        if (per) {
+            b %= n;
+            if (b < 0) b += n;
+        }
+        if (finite && (per || (b >= 1 && b + 3 <= n - 2))) base = b;
     }
     const int w0 = (threadIdx.x & 31) & ~(LANES - 1);
-    NodeStencil S;
+    NodeStencil<T> S;
     S.ok = true;
     // every lane executes every full-mask shuffle (no short-circuit around
     // them: a lane that skipped one would leave the others waiting)
     for (int a = 0; a < 3; ++a) {
         S.base[a] = __shfl_sync(0xffffffffu, base, w0 + a);
-        S.frac[a] = __shfl_sync(0xffffffffu, fr, w0 + a);
-        const int ok_a = __shfl_sync(0xffffffffu, ok ? 1 : 0, w0 + a);
-        S.ok = S.ok && (ok_a != 0);
+        S.f[a] = __shfl_sync(0xffffffffu, f, w0 + a);
+        S.s[a] = __shfl_sync(0xffffffffu, s, w0 + a);
+        if constexpr (DERIV) S.ds[a] = __shfl_sync(0xffffffffu, ds, w0 + a);
+        S.ok = S.ok && S.base[a] != kNone;
     }
     return S;
 }
 
-// Weights of the lane's x-row (w[0..3]) and of its y and z rows, in the
-// storage precision: offsets frac + (1 - k); in FP32 the fraction is
-// rounded to float first, in FP64 the offsets are the correctly rounded
-// r - (base + k).
+// The weight of point k (0..3) along an axis, and its derivative in r.
 template <typename T>
-__device__ __forceinline__ void stencil_weights(const NodeStencil &S, int b, int c, T w[4], T &wy, T &wz)
+__device__ __forceinline__ T stencil_w(const T f, const T s, const int k)
 {
-    if constexpr (sizeof(T) == 8) {
-        for (int a = 0; a < 4; ++a) w[a] = peskin_phi<T>(S.frac[0] + (double)(1 - a));
-        wy = peskin_phi<T>(S.frac[1] + (double)(1 - b));
-        wz = peskin_phi<T>(S.frac[2] + (double)(1 - c));
-    } else {
-        const T fx = T(S.frac[0]), fy = T(S.frac[1]), fz = T(S.frac[2]);
-        for (int a = 0; a < 4; ++a) w[a] = peskin_phi<T>(fx + T(1 - a));
-        wy = peskin_phi<T>(fy + T(1 - b));
-        wz = peskin_phi<T>(fz + T(1 - c));
-    }
+    return T(0.125) * ((k < 2 ? T(3) - T(2) * f : T(1) + T(2) * f) + ((k == 1 || k == 2) ? s : -s));
+}
+template <typename T>
+__device__ __forceinline__ T stencil_dw(const T ds, const int k)
+{
+    return T(0.125) * ((k < 2 ? T(-2) : T(2)) + ((k == 1 || k == 2) ? ds : -ds));
+}
+// Lattice index of point k along an axis of n nodes: only a periodic stencil
+// passes the end, once.
+__device__ __forceinline__ int stencil_at(const int base, const int k, const int n)
+{
+    const int g = base + k;
+    return g >= n ? g - n : g;
 }
 
 // n / d for 0 <= n < 2^31, d >= 2 (see DivBy).
@@ -340,37 +333,11 @@ __device__ __forceinline__ bool node_in_patch(const LbView &L, const Ctl *c, int
            (unsigned)dz <= (unsigned)c->patch_ext[buf][2];
 }
 
-// Surface-tension force of triangle t on its vertex in position `slot`
-// (Eq. (pi_drop), F_i = -sigma dA/dx_i summed over the triangles around i):
-// m_t x (x_{slot+2} - x_{slot+1}) with the scaled unit normal
-// m_t = -sigma/2 N/|N|, N = (x1 - x0) x (x2 - x0).  Positions are FP64; the
-// edge vectors are formed in FP64 and the rest runs in G (the step uses
-// FP64 mesh geometry for either population precision).
-template <typename G>
-__device__ __forceinline__ void tri_force(const MeshView &M, const int t, const int slot, G g[3])
-{
-    double x[3][3];
-    for (int k = 0; k < 3; ++k) {
-        const int v = M.tris[3 * t + k];
-        for (int a = 0; a < 3; ++a) x[k][a] = M.r[3 * v + a];
-    }
-    G e1[3], e2[3], N[3];
-    for (int a = 0; a < 3; ++a) {
-        e1[a] = G(x[1][a] - x[0][a]);
-        e2[a] = G(x[2][a] - x[0][a]);
-    }
-    cross3(e1, e2, N);
-    const G s = G(-0.5) * G(M.sigma) * rsqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
-    const G m[3] = {s * N[0], s * N[1], s * N[2]};
-    const int kp = slot == 2 ? 0 : slot + 1, km = slot == 0 ? 2 : slot - 1;
-    const G dd[3] = {G(x[km][0] - x[kp][0]), G(x[km][1] - x[kp][1]), G(x[km][2] - x[kp][2])};
-    cross3(m, dd, g);
-}
-
-// The same force in two stages, so that the FP64 normal of each triangle is
-// evaluated once per step instead of once per corner: tri_moment gives m_t
-// = -sigma N_t / (2 |N_t|) (the m of tri_force<double>, bit for bit), and
-// tri_force_m the force on corner `slot` from a stored m_t.
+// Surface-tension force of a triangle on its vertex x_i (Eq. (pi_drop), F_i =
+// -sigma dA/dx_i summed over the triangles around i): m x (q - p) for the
+// other two vertices p, q in the triangle's order, with m = -sigma N / (2
+// |N|), N its normal.  FP64 mesh geometry for either population precision.
+// tri_moment evaluates m once per triangle for the ensemble's force kernel.
 template <class P>
 __device__ __forceinline__ void tri_moment(const MeshView &M, const int t, double m[3], const P &K)
 {
@@ -387,17 +354,6 @@ __device__ __forceinline__ void tri_moment(const MeshView &M, const int t, doubl
     cross3(e1, e2, N);
     const double s = -0.5 * M.sigma * rsqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
     for (int a = 0; a < 3; ++a) m[a] = s * N[a];
-}
-
-template <class P>
-__device__ __forceinline__ void tri_force_m(const MeshView &M, const int t, const int slot, const double m[3],
-                                            double g[3], const P &K)
-{
-    const int kp = slot == 2 ? 0 : slot + 1, km = slot == 0 ? 2 : slot - 1;
-    const int vp = K.ld(M.tris + 3 * t + kp), vm = K.ld(M.tris + 3 * t + km);
-    double dd[3];
-    for (int a = 0; a < 3; ++a) dd[a] = K.ld(M.r + 3 * vm + a) - K.ld(M.r + 3 * vp + a);
-    cross3(m, dd, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -440,40 +396,70 @@ __device__ double block_max(double v, double *sh)
     return out;
 }
 
+// Bits of a non-negative double, which order as the values do; NaN counts as 0
+// (fmax skips it).
+__device__ __forceinline__ unsigned long long order_bits(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return b > 0x7ff0000000000000ull ? 0ull : b;
+}
+// Order-preserving key of any double (NaN: 0 under a maximum).
+__device__ __forceinline__ unsigned long long order_key(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if ((b & 0x7fffffffffffffffull) > 0x7ff0000000000000ull) return 0ull;
+    return (b >> 63) ? ~b : b | 0x8000000000000000ull;
+}
+__device__ __forceinline__ double key_value(unsigned long long k)
+{
+    return __longlong_as_double((long long)((k >> 63) ? k & 0x7fffffffffffffffull : ~k));
+}
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v)
+{
+    const unsigned hi = (unsigned)(v >> 32);
+    const unsigned top = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = __reduce_max_sync(0xffffffffu, hi == top ? (unsigned)v : 0u);
+    return ((unsigned long long)top << 32) | lo;
+}
+
 // Patch of lattice nodes the droplet's stencils can touch, from the node
 // bounding box [mn, mx]: floor(mn)-1 .. floor(mx)+2 per axis (periodic axes
 // keep the lower corner inside the box and may wrap; Zou-He axes clamp).
 // `grow` extra nodes on each side (1 covers the nodes' motion over one more
 // step: |u| <= 0.3 keeps floor(r) within one node).
+__device__ __forceinline__ void write_patch_axis(const LbView &L, const int a, const double lo_d, const double hi_d,
+                                                 const int buf, const int grow)
+{
+    const int n = a == 0 ? L.n[0] : (a == 1 ? L.n[1] : L.n[2]);
+    const int bc = a == 0 ? L.bc[0] : (a == 1 ? L.bc[1] : L.bc[2]);
+    int *const plo = &L.ctl->patch_lo[buf][a], *const pext = &L.ctl->patch_ext[buf][a];
+    if (!(lo_d > -1e8 && lo_d < 1e8) || !(hi_d > -1e8 && hi_d < 1e8) || hi_d < lo_d) {
+        *plo = 0;
+        *pext = n - 1;
+        return;
+    }
+    int lo = __double2int_rd(lo_d) - 1 - grow, hi = __double2int_rd(hi_d) + 2 + grow;
+    if (bc == IBL_BC_PERIODIC) {
+        if (hi - lo + 1 >= n) {
+            lo = 0;
+            hi = n - 1;
+        } else {
+            int l2 = lo % n;
+            if (l2 < 0) l2 += n;
+            hi = l2 + (hi - lo);
+            lo = l2;
+        }
+    } else {
+        if (lo < 0) lo = 0;
+        if (hi > n - 1) hi = n - 1;
+        if (hi < lo) hi = lo;
+    }
+    *plo = lo;
+    *pext = hi - lo;
+}
 __device__ void write_patch(const LbView &L, const double mn[3], const double mx[3], int buf, int grow)
 {
-    for (int a = 0; a < 3; ++a) {
-        const int n = L.n[a];
-        double lo_d = mn[a], hi_d = mx[a];
-        if (!(lo_d > -1e8 && lo_d < 1e8) || !(hi_d > -1e8 && hi_d < 1e8) || hi_d < lo_d) {
-            L.ctl->patch_lo[buf][a] = 0;
-            L.ctl->patch_ext[buf][a] = n - 1;
-            continue;
-        }
-        long long lo = (long long)floor(lo_d) - 1 - grow, hi = (long long)floor(hi_d) + 2 + grow;
-        if (L.bc[a] == IBL_BC_PERIODIC) {
-            if (hi - lo + 1 >= n) {
-                lo = 0;
-                hi = n - 1;
-            } else {
-                long long l2 = lo % n;
-                if (l2 < 0) l2 += n;
-                hi = l2 + (hi - lo);
-                lo = l2;
-            }
-        } else {
-            if (lo < 0) lo = 0;
-            if (hi > n - 1) hi = n - 1;
-            if (hi < lo) hi = lo;
-        }
-        L.ctl->patch_lo[buf][a] = (int)lo;
-        L.ctl->patch_ext[buf][a] = (int)(hi - lo);
-    }
+    for (int a = 0; a < 3; ++a) write_patch_axis(L, a, mn[a], mx[a], buf, grow);
 }
 
 __device__ void block_bbox_patch(const LbView &L, const MeshView &M, const double *r, int nv, int buf)

@@ -198,14 +198,6 @@ __device__ __forceinline__ void bc_dispatch(T (&f)[19], const T (&uw)[3], int ru
 // without the Guo source.
 enum { LAT_FULL = 0, LAT_FAR = 1, LAT_NEAR = 2 };
 
-// Population access: slot i of the node at byte offset `off` of its array.
-// The array's base is the same for all threads, the offset 32 bits.
-template <typename T>
-__device__ __forceinline__ T *slot_at(T *f, const int i, const long long qs, const unsigned off)
-{
-    return reinterpret_cast<T *>(reinterpret_cast<char *>(f + i * qs) + off);
-}
-
 // 3 w_i, the weight of the odd (momentum) parts of the equilibrium and of
 // the Guo source.  The exact values are 1/6 (|c_i|^2 = 1) and 1/12 (|c_i|^2
 // = 2), and sum_i c_ia c_ia 3 w_i = 2/6 + 8/12 = 1 carries the momentum
@@ -718,8 +710,11 @@ __global__ void __launch_bounds__(NT, (B > 768 / NT ? B : 768 / NT)) k_lattice_s
 }
 
 // The patch nodes of the step: one warp per row (y, z) of the patch box,
-// its lanes along x (32 at a time), rows grid-strided over the warps of the
-// grid, so that each access of a warp is one contiguous run of a row.
+// its lanes along x (32 at a time), so that each access of a warp is one
+// contiguous run of a row.  Rows go round the blocks before a block gets its
+// second one: a patch of fewer rows than the grid has warps (324 of 2432 for a
+// 32^3 box) otherwise runs on the SMs of the first blocks alone, eight warps
+// deep in each SM's FP64 pipe.
 template <typename T, bool ODD, bool REC, bool PER, class P>
 __device__ __forceinline__ void patch_rows(const LbView &L, const int buf, const int warp0, const int nwarps)
 {
@@ -750,7 +745,7 @@ template <typename T, bool ODD, bool REC, bool PER>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lattice_near(LbView L, int buf)
 {
     const int wpb = blockDim.x >> 5;
-    patch_rows<T, ODD, REC, PER, L2Keep>(L, buf, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb);
+    patch_rows<T, ODD, REC, PER, L2Keep>(L, buf, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * wpb);
 }
 
 // Ensemble: the nodes outside each member's droplet patch, one launch over
@@ -805,7 +800,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_lattice_near_ba
                                                                                     const int buf)
 {
     const int wpb = blockDim.x >> 5;
-    patch_rows<T, ODD, false, PER, P>(G.v[blockIdx.y], buf, blockIdx.x * wpb + (threadIdx.x >> 5), gridDim.x * wpb);
+    patch_rows<T, ODD, false, PER, P>(G.v[blockIdx.y], buf, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * wpb);
 }
 
 
@@ -834,28 +829,50 @@ __global__ void __launch_bounds__(256) k_init(LbView L)
 
 // ---------------------------------------------------------------------------
 // Immersed boundary.
-// Warp 0 of block 0 of the force/spread kernel of step t: reduce the
-// bounding-box rows of r_t left by the previous interpolation (or
-// regularisation) into the patch of step t + 1, grown by one node, in
-// buffer `buf` (the parity of step t + 1).
+// One block beside the force/spread kernel of step t: reduce the bounding-box
+// rows of r_t left by the previous interpolation (or regularisation) into the
+// patch of step t + 1, grown by one node, in buffer `buf` (the parity of step
+// t + 1).  Minima and maxima are integer ones on order-preserving keys: in
+// FP64, by one warp before its share of the nodes, they were the longest chain
+// of the kernel (a warp's FP64 instruction takes 64 cycles).
 template <class P>
-__device__ void patch_from_rows(const LbView &L, const MeshView &M, int buf)
+__device__ __forceinline__ void patch_from_rows(const LbView &L, const MeshView &M, const int buf)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ unsigned long long box[4][6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = L.ctl->n_part;
     const P K;
-    double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-    for (int k = lane; k < rows; k += 32)
-        for (int a = 0; a < 3; ++a) {
-            mn[a] = fmin(mn[a], K.ld(M.part + 6 * k + a));
-            mx[a] = fmax(mx[a], K.ld(M.part + 6 * k + 3 + a));
+    unsigned long long v[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+    for (int k = threadIdx.x; k < rows; k += kIbThreads)
+        for (int a = 0; a < 6; ++a) {
+            // minima as maxima of the negated value (sign bit)
+            const double x = K.ld(M.part + 6 * k + a);
+            const double y = a < 3 ? __longlong_as_double(__double_as_longlong(x) ^ 0x8000000000000000ull) : x;
+            v[a] = max(v[a], order_key(y));
         }
-    for (int a = 0; a < 3; ++a)
-        for (int o = 16; o > 0; o >>= 1) {
-            mn[a] = fmin(mn[a], __shfl_xor_sync(0xffffffffu, mn[a], o));
-            mx[a] = fmax(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], o));
+    for (int a = 0; a < 6; ++a) {
+        const unsigned long long m = warp_max(v[a]);
+        if (lane == 0) box[warp][a] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        unsigned long long lo = 0ull, hi = 0ull;
+        for (int w = 0; w < kIbThreads / 32; ++w) {
+            lo = max(lo, box[w][a]);
+            hi = max(hi, box[w][3 + a]);
         }
-    if (lane == 0) write_patch(L, mn, mx, buf, 1);
+        write_patch_axis(L, a, lo ? -key_value(lo) : 1e300, hi ? key_value(hi) : -1e300, buf, 1);
+    }
+    if (M.rec_ctl && threadIdx.x == 32) {
+        // this step's patch buffer, for the adjoint
+        const int pb = (buf + 2) % 3;
+        for (int a = 0; a < 4; ++a) {
+            M.rec_ctl->patch_lo[pb][a] = L.ctl->patch_lo[pb][a];
+            M.rec_ctl->patch_ext[pb][a] = L.ctl->patch_ext[pb][a];
+        }
+    }
+    __syncthreads();  // the block's next unit of work may reuse the rows
 }
 
 // Nodal force F_i = -sigma dA/dx_i (Eq. (pi_drop)) gathered over the
@@ -864,13 +881,12 @@ __device__ void patch_from_rows(const LbView &L, const MeshView &M, int buf)
 // lanes per node: the lanes split the incident triangles (reduced with
 // shuffles), then each lane adds 16 / LANES x-rows of four stencil points.
 // STORED: m_t comes from M.tm (written by k_tri_moment_batched just before);
-// otherwise each lane evaluates it for its triangle (three times per
-// triangle in all, but one kernel boundary fewer on the droplet chain of a
-// single droplet, which is latency bound).
+// otherwise each lane evaluates it for its triangle, from the edges out of its
+// node (three times per triangle in all, but one kernel boundary fewer on the
+// droplet chain of a single droplet, which is latency bound).
 template <typename T, bool STORED, int LANES, class P = L2Keep>
-__device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, const int blk, const int next_buf)
+__device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, const int blk)
 {
-    if (blk == 0 && threadIdx.x < 32) patch_from_rows<P>(L, M, next_buf);
     const int gid = blk * (kIbThreads / LANES) + threadIdx.x / LANES;
     const int lane = threadIdx.x % LANES;
     const bool valid = gid < M.nv;
@@ -878,60 +894,64 @@ __device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, 
     const P K;
     double F[3] = {0.0, 0.0, 0.0};
     const int k0 = K.ld(M.n2t_ptr + i), k1 = K.ld(M.n2t_ptr + i + 1);
+    double ra;
+    const NodeStencil<T> S = node_stencil<T, LANES, false>(L, M.r + 3 * i, lane, K, ra);
+    double xi[3];
+    if constexpr (!STORED)
+        for (int a = 0; a < 3; ++a) xi[a] = K.ld(M.r + 3 * i + a);
     for (int k = k0 + lane; k < k1; k += LANES) {
         const int e = K.ld(M.n2t + k);
-        const int t = e / 3;
-        double m[3];
+        const int t = e / 3, slot = e - 3 * t;
+        const int vp = K.ld(M.tris + (slot == 2 ? e - 2 : e + 1)), vq = K.ld(M.tris + (slot == 0 ? e + 2 : e - 1));
+        double p[3], q[3];
+        for (int a = 0; a < 3; ++a) p[a] = K.ld(M.r + 3 * vp + a);
+        for (int a = 0; a < 3; ++a) q[a] = K.ld(M.r + 3 * vq + a);
+        double m[3], g[3];
         if constexpr (STORED) {
             for (int a = 0; a < 3; ++a) m[a] = K.ld(M.tm + 3 * t + a);
         } else {
-            tri_moment(M, t, m, K);
+            const double e1[3] = {p[0] - xi[0], p[1] - xi[1], p[2] - xi[2]};
+            const double e2[3] = {q[0] - xi[0], q[1] - xi[1], q[2] - xi[2]};
+            double N[3];
+            cross3(e1, e2, N);
+            const double s = -0.5 * M.sigma * rsqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
+            for (int a = 0; a < 3; ++a) m[a] = s * N[a];
         }
-        double g[3];
-        tri_force_m(M, t, e - 3 * t, m, g, K);
+        const double dd[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
+        cross3(m, dd, g);
         for (int a = 0; a < 3; ++a) F[a] += g[a];
     }
     for (int o = LANES / 2; o > 0; o >>= 1)
         for (int a = 0; a < 3; ++a) F[a] += __shfl_xor_sync(0xffffffffu, F[a], o, LANES);
-    if (valid && lane == 0) {
-        M.fn[3 * i] = F[0];
-        M.fn[3 * i + 1] = F[1];
-        M.fn[3 * i + 2] = F[2];
-        if (M.rec_r) {
-            M.rec_r[3 * i] = M.r[3 * i];
-            M.rec_r[3 * i + 1] = M.r[3 * i + 1];
-            M.rec_r[3 * i + 2] = M.r[3 * i + 2];
-        }
+    if (valid && lane < 3) {
+        M.fn[3 * i + lane] = lane == 0 ? F[0] : (lane == 1 ? F[1] : F[2]);
+        if (M.rec_r) M.rec_r[3 * i + lane] = ra;
     }
-    if (M.rec_ctl && blk == 0 && threadIdx.x == 32) {
-        // this step's patch buffer; warp 0 writes the next step's
-        const int pb = (next_buf + 2) % 3;
-        for (int a = 0; a < 4; ++a) {
-            M.rec_ctl->patch_lo[pb][a] = L.ctl->patch_lo[pb][a];
-            M.rec_ctl->patch_ext[pb][a] = L.ctl->patch_ext[pb][a];
-        }
-    }
-    const NodeStencil S = node_stencil<LANES, P>(L, M.r + 3 * i, lane, &K);
     if (valid && !S.ok && lane == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_WALL);
     if (!valid || !S.ok) return;
-    const bool perx = L.bc[0] == IBL_BC_PERIODIC, pery = L.bc[1] == IBL_BC_PERIODIC,
-               perz = L.bc[2] == IBL_BC_PERIODIC;
     const int nx = L.n[0], nxy = L.n[0] * L.n[1];
     T *force = static_cast<T *>(L.force);  // [nodes][4]
     const T Fx = T(F[0]), Fy = T(F[1]), Fz = T(F[2]);
-    // the lane's (y, z) rows r = lane, lane + LANES, ...: (b, c) = (r & 3, r >> 2)
+    T w[4];
+    int x[4];
 #pragma unroll
-    for (int q = 0; q < 16 / LANES; ++q) {
-        const int r = lane + LANES * q, b = r & 3, c = r >> 2;
-        T w[4], wy, wz;
-        stencil_weights<T>(S, b, c, w, wy, wz);
-        const int row =
-            wrap_index(S.base[1] + b, L.n[1], pery) * nx + wrap_index(S.base[2] + c, L.n[2], perz) * nxy;
+    for (int a = 0; a < 4; ++a) {
+        w[a] = stencil_w(S.f[0], S.s[0], a);
+        x[a] = stencil_at(S.base[0], a, nx);
+    }
+    // the lane's (y, z) rows r = lane, lane + LANES, ...: (b, c) = (r & 3, r >> 2)
+    const int b = lane & 3;
+    const T wy = stencil_w(S.f[1], S.s[1], b);
+    const int y = stencil_at(S.base[1], b, L.n[1]) * nx;
+#pragma unroll
+    for (int k = 0; k < 16 / LANES; ++k) {
+        const int c = (lane >> 2) + (LANES / 4) * k;
+        const T wz = stencil_w(S.f[2], S.s[2], c);
+        const int row = y + stencil_at(S.base[2], c, L.n[2]) * nxy;
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const T dl = w[a] * wy * wz;
-            const int id = row + wrap_index(S.base[0] + a, nx, perx);
-            K.red_add3(force + 4 * id, Fx * dl, Fy * dl, Fz * dl);
+            K.red_add3(slot_at(force, 0, 0, (unsigned)(row + x[a]) * (unsigned)(4 * sizeof(T))), Fx * dl, Fy * dl, Fz * dl);
         }
     }
 }
@@ -954,9 +974,12 @@ __global__ void __launch_bounds__(128) k_tri_moment_batched(const __grid_constan
 template <typename T, int LANES>
 __global__ void __launch_bounds__(128) k_spread(LbView L, MeshView M, int next_buf, int nblk)
 {
-    // node groups block-strided: a grid capped below nblk leaves SM slots to
-    // the concurrent outside update
-    for (int b = blockIdx.x; b < nblk; b += (int)gridDim.x) spread_body<T, false, LANES>(L, M, b, next_buf);
+    // the first block reduces the patch; node groups are block-strided over the others
+    if (blockIdx.x == 0) {
+        patch_from_rows<L2Keep>(L, M, next_buf);
+        return;
+    }
+    for (int b = (int)blockIdx.x - 1; b < nblk; b += (int)gridDim.x - 1) spread_body<T, false, LANES>(L, M, b);
 }
 
 // Re-centring (Sec. 3.2: the linearisation is centred on the droplet's
@@ -1085,27 +1108,33 @@ __device__ __forceinline__ void interp_body(const LbView &L, const MeshView &M, 
     const bool valid = gid < M.nv;
     const int i = valid ? gid : M.nv - 1;
     const P K;
-    const NodeStencil S = node_stencil<LANES, P>(L, M.r + 3 * i, lane, &K);
+    double r;  // the lane's coordinate (lanes 0..2)
+    const NodeStencil<T> S = node_stencil<T, LANES, false>(L, M.r + 3 * i, lane, K, r);
     T v[3] = {T(0), T(0), T(0)};
     if (S.ok) {
-        const bool perx = L.bc[0] == IBL_BC_PERIODIC, pery = L.bc[1] == IBL_BC_PERIODIC,
-                   perz = L.bc[2] == IBL_BC_PERIODIC;
         const int nx = L.n[0], nxy = L.n[0] * L.n[1];
-        const T *vel = static_cast<const T *>(L.vel);  // [nodes][4]
-        // the lane's (y, z) rows r = lane, lane + LANES, ...: (b, c) = (r & 3, r >> 2)
+        T *vel = static_cast<T *>(L.vel);  // [nodes][4]
+        T w[4];
+        int x[4];
 #pragma unroll
-        for (int q = 0; q < 16 / LANES; ++q) {
-            const int r = lane + LANES * q, b = r & 3, c = r >> 2;
-            T w[4], wy, wz;
-            stencil_weights<T>(S, b, c, w, wy, wz);
-            const int row =
-                wrap_index(S.base[1] + b, L.n[1], pery) * nx + wrap_index(S.base[2] + c, L.n[2], perz) * nxy;
+        for (int a = 0; a < 4; ++a) {
+            w[a] = stencil_w(S.f[0], S.s[0], a);
+            x[a] = stencil_at(S.base[0], a, nx);
+        }
+        // the lane's (y, z) rows r = lane, lane + LANES, ...: (b, c) = (r & 3, r >> 2)
+        const int b = lane & 3;
+        const T wy = stencil_w(S.f[1], S.s[1], b);
+        const int y = stencil_at(S.base[1], b, L.n[1]) * nx;
+#pragma unroll
+        for (int k = 0; k < 16 / LANES; ++k) {
+            const int c = (lane >> 2) + (LANES / 4) * k;
+            const T wz = stencil_w(S.f[2], S.s[2], c);
+            const int row = y + stencil_at(S.base[2], c, L.n[2]) * nxy;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
                 const T dl = w[a] * wy * wz;
-                const int id = row + wrap_index(S.base[0] + a, nx, perx);
                 T ua, ub, uc;
-                K.ld3(vel + 4 * id, ua, ub, uc);
+                K.ld3(slot_at(vel, 0, 0, (unsigned)(row + x[a]) * (unsigned)(4 * sizeof(T))), ua, ub, uc);
                 v[0] += ua * dl;
                 v[1] += ub * dl;
                 v[2] += uc * dl;
@@ -1114,52 +1143,41 @@ __device__ __forceinline__ void interp_body(const LbView &L, const MeshView &M, 
     }
     for (int o = LANES / 2; o > 0; o >>= 1)
         for (int a = 0; a < 3; ++a) v[a] += __shfl_xor_sync(0xffffffffu, v[a], o, LANES);
-    const bool have = valid && lane == 0;
-    double r[3] = {0.0, 0.0, 0.0};
-    if (have) {
-        r[0] = K.ld(M.r + 3 * i);
-        r[1] = K.ld(M.r + 3 * i + 1);
-        r[2] = K.ld(M.r + 3 * i + 2);
-        if (!S.ok) {
+    // forward Euler, one component a lane; floor of the new coordinate for
+    // the bounding box, whose patch only needs floors (conversion saturates:
+    // a coordinate beyond 2^31 makes the patch the whole axis, as any beyond
+    // 1e8 does; NaN is left out)
+    constexpr int kHigh = 2147483647, kLow = -2147483647 - 1;
+    int lo = kHigh, hi = kLow;
+    if (valid && lane < 3) {
+        if (S.ok) {
+            r += (double)(lane == 0 ? v[0] : (lane == 1 ? v[1] : v[2]));
+            K.st(M.r + 3 * i + lane, r);
+        } else if (lane == 0) {
             atomicOr(&L.ctl->err, IBL_ERRBIT_WALL);
-        } else {
-            r[0] += (double)v[0];
-            r[1] += (double)v[1];
-            r[2] += (double)v[2];
-            K.st(M.r + 3 * i, r[0]);
-            K.st(M.r + 3 * i + 1, r[1]);
-            K.st(M.r + 3 * i + 2, r[2]);
         }
+        if (r == r) lo = hi = __double2int_rd(r);
     }
-    // block min / max of the new positions -> one partial row per block; the
-    // next force/spread kernel reduces the rows into the patch (no tail here)
-    __shared__ double smn[3][4], smx[3][4];
-    const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // block min / max -> one partial row per block; the next force/spread
+    // kernel reduces the rows into the patch (no tail here)
+    __shared__ int box[kIbThreads / 32][6];
+    const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int a = 0; a < 3; ++a) {
-        // lanes 0, LANES, 2 LANES, ... hold the warp's nodes
-        double mn = have ? r[a] : 1e300, mx = have ? r[a] : -1e300;
-        for (int o = LANES; o < 32; o <<= 1) {
-            mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        }
+        const int mn = __reduce_min_sync(0xffffffffu, lane == a ? lo : kHigh);
+        const int mx = __reduce_max_sync(0xffffffffu, lane == a ? hi : kLow);
         if (wlane == 0) {
-            smn[a][warp] = mn;
-            smx[a][warp] = mx;
+            box[warp][a] = mn;
+            box[warp][3 + a] = mx;
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int a = 0; a < 3; ++a) {
-            double mn = smn[a][0], mx = smx[a][0];
-            for (int w = 1; w < nw; ++w) {
-                mn = fmin(mn, smn[a][w]);
-                mx = fmax(mx, smx[a][w]);
-            }
-            K.st(M.part + 6 * blk + a, mn);
-            K.st(M.part + 6 * blk + 3 + a, mx);
-        }
-        if (blk == 0) L.ctl->n_part = nblk;
+    if (threadIdx.x < 6) {
+        const int a = threadIdx.x;
+        int m = box[0][a];
+        for (int w = 1; w < kIbThreads / 32; ++w) m = a < 3 ? min(m, box[w][a]) : max(m, box[w][a]);
+        K.st(M.part + 6 * blk + a, (double)m);
     }
+    if (blk == 0 && threadIdx.x == 0) L.ctl->n_part = nblk;
 }
 
 template <typename T, int LANES>
@@ -1181,12 +1199,18 @@ __global__ void __launch_bounds__(128) k_interp(LbView L, MeshView M, int nblk)
 template <typename T, class P>
 __global__ void __launch_bounds__(128)
     k_spread_batched(const __grid_constant__ LbGroup LG, const __grid_constant__ MeshGroup MG, const int m0,
-                     const int b0, const int nb, const int *__restrict__ blk_member,
+                     const int nm, const int b0, const int nb, const int *__restrict__ blk_member,
                      const int *__restrict__ blk_start, const int next_buf)
 {
-    for (int bb = b0 + (int)blockIdx.x; bb < b0 + nb; bb += (int)gridDim.x) {
+    // first the patches of the group's nm members, then the node groups
+    for (int u = (int)blockIdx.x; u < nm + nb; u += (int)gridDim.x) {
+        if (u < nm) {
+            patch_from_rows<P>(LG.v[u], MG.v[u], next_buf);
+            continue;
+        }
+        const int bb = b0 + u - nm;
         const int mi = blk_member[bb];
-        spread_body<T, true, kFwdLanes, P>(LG.v[mi - m0], MG.v[mi - m0], bb - blk_start[mi], next_buf);
+        spread_body<T, true, kFwdLanes, P>(LG.v[mi - m0], MG.v[mi - m0], bb - blk_start[mi]);
     }
 }
 
@@ -1549,7 +1573,7 @@ cudaError_t launch_spread(const LbView &L, const MeshView &M, int next_buf, cuda
 {
     const int lanes = fwd_lanes(M);
     const int nblk = (int)blocks_for((long long)M.nv * lanes, kIbThreads);
-    const dim3 g(ib_grid(nblk)), b(kIbThreads);
+    const dim3 g(1 + ib_grid(nblk)), b(kIbThreads);  // and the patch block
     if (lanes == 16) {
         if (L.precision == IBL_FP64) return launch_p(k_spread<double, 16>, g, b, s, prio, L, M, next_buf, nblk);
         return launch_p(k_spread<float, 16>, g, b, s, prio, L, M, next_buf, nblk);
@@ -1649,13 +1673,13 @@ static cudaError_t ensemble_pre_t(const EnsembleView &E, int m0, int m1, int pbu
     }
     if (e == cudaSuccess) e = launch_p(k_tri_moment_batched<P>, dim3(tb, m1 - m0), dim3(128), s, prio, G.mg);
     const int nb0 = E.node_start[m0], nb = E.node_start[m1] - nb0;
-    const dim3 g(chain_grid(E, nb));
+    const dim3 g(chain_grid(E, nb + m1 - m0));
     if (e == cudaSuccess) {
         if (E.precision == IBL_FP64)
-            e = launch_p(k_spread_batched<double, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, nb0, nb,
+            e = launch_p(k_spread_batched<double, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, m1 - m0, nb0, nb,
                          E.node_member, E.node_start_d, nxt);
         else
-            e = launch_p(k_spread_batched<float, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, nb0, nb,
+            e = launch_p(k_spread_batched<float, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, m1 - m0, nb0, nb,
                          E.node_member, E.node_start_d, nxt);
     }
     return e;

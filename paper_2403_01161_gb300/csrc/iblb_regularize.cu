@@ -203,32 +203,6 @@ __device__ __forceinline__ double cluster_ld(unsigned a)
     return v;
 }
 
-// Bits of a non-negative double, which order as the values do; NaN counts as 0
-// (fmax skips it).
-__device__ __forceinline__ unsigned long long order_bits(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return b > 0x7ff0000000000000ull ? 0ull : b;
-}
-// Order-preserving key of any double (NaN: 0 under a maximum).
-__device__ __forceinline__ unsigned long long order_key(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    if ((b & 0x7fffffffffffffffull) > 0x7ff0000000000000ull) return 0ull;
-    return (b >> 63) ? ~b : b | 0x8000000000000000ull;
-}
-__device__ __forceinline__ double key_value(unsigned long long k)
-{
-    return __longlong_as_double((long long)((k >> 63) ? k & 0x7fffffffffffffffull : ~k));
-}
-__device__ __forceinline__ unsigned long long warp_max(unsigned long long v)
-{
-    const unsigned hi = (unsigned)(v >> 32);
-    const unsigned top = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned lo = __reduce_max_sync(0xffffffffu, hi == top ? (unsigned)v : 0u);
-    return ((unsigned long long)top << 32) | lo;
-}
-
 // Sum over the block, left in every thread of warp 0.
 template <int K>
 __device__ __forceinline__ void reg_block_sum(double (&v)[K], double (*sh)[K])
