@@ -74,7 +74,7 @@ bool lb_layout(const ibl_lb_params *p, int n_frames, Layout &L)
 
 struct MeshLayout {
     size_t r = 0, fn = 0, tris = 0, n2t_ptr = 0, n2t = 0, nb_ptr = 0, nb_idx = 0, s0 = 0, s1 = 0, s2 = 0,
-           tm = 0, part = 0, cpart = 0, obs_part = 0, ring = 0, total = 0;
+           tm = 0, part = 0, unused = 0, obs_part = 0, ring = 0, total = 0;
 };
 
 bool mesh_layout(int nv, int nt, MeshLayout &L)
@@ -98,7 +98,7 @@ bool mesh_layout(int nv, int nt, MeshLayout &L)
     L.s2 = take(sizeof(double) * 3 * nv);
     L.tm = take(sizeof(double) * 3 * nt);
     L.part = take(sizeof(double) * 6 * (((size_t)nv + 7) / 8 + 1));  // one row per interpolation block
-    L.cpart = take(sizeof(double) * 4 * iblb::kCentreBlocks);
+    L.unused = take(sizeof(double) * 64);  // keeps the offsets of saved states
     L.obs_part = take(sizeof(double) * 11 * iblb::kObsBlocksMax);
     L.ring = take(sizeof(ibl_observables) * iblb::kRingCap);
     L.total = off;
@@ -299,22 +299,15 @@ int one_step(ibl_lb *lb, bool record, cudaStream_t sL, cudaStream_t sH)
         lb->host_step = next;
         return IBL_OK;
     }
-    // helper stream: forces + spread (and the next step's patch), then the
-    // patch nodes once the previous outside update has finished
-    // with re-centring, first the step's centre (from the positions the
-    // previous step left), which the outside update reads on its faces
+    // helper stream: forces + spread (and the next step's patch; with
+    // re-centring the step's centre, which the outside update reads on its
+    // faces; with a viscosity ratio the inside flags of the patch nodes), then
+    // the patch nodes once the previous outside update has finished
     cudaEvent_t evCentre = lb->capturing ? lb->cCentre : lb->evCentre;
-    e = cudaSuccess;
-    if (lb->v.recentre) {
-        e = iblb::launch_centre(lb->v, m->v, pbuf, sH, lb->hi_prio);
-        if (e == cudaSuccess) e = cudaEventRecord(evCentre, sH);
-    }
-    // with a viscosity ratio, the inside flags of this step's patch nodes
-    // (read and cleared by the patch update below)
-    if (e == cudaSuccess && lb->v.visc) e = iblb::launch_indicator(lb->v, m->v, pbuf, sH, lb->hi_prio);
     const int ps = prof_begin(lb, PROF_SPREAD, sH);
-    if (e == cudaSuccess) e = iblb::launch_spread(lb->v, m->v, pnext, sH, lb->hi_prio);
+    e = iblb::launch_spread(lb->v, m->v, pnext, sH, lb->hi_prio);
     prof_end(lb, ps, sH);
+    if (e == cudaSuccess && lb->v.recentre) e = cudaEventRecord(evCentre, sH);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(sH, evFar[par ^ 1], 0);
     if (e == cudaSuccess) e = iblb::launch_near(lb->v, odd, record, pbuf, sH, lb->hi_prio);
     if (e == cudaSuccess) e = cudaEventRecord(evNear[par], sH);
@@ -551,7 +544,6 @@ int mesh_attach(ibl_lb *lb, int nv, const double *r, int nt, const int *tri_in, 
     m->v.s2 = reinterpret_cast<double *>(w + L.s2);
     m->v.tm = reinterpret_cast<double *>(w + L.tm);
     m->v.part = reinterpret_cast<double *>(w + L.part);
-    m->v.cpart = reinterpret_cast<double *>(w + L.cpart);
     m->v.obs_part = reinterpret_cast<double *>(w + L.obs_part);
     m->v.ring = reinterpret_cast<ibl_observables *>(w + L.ring);
     m->v.ring_cap = iblb::kRingCap;
@@ -937,8 +929,9 @@ int ensemble_one_step(ibl_ensemble *e, cudaStream_t sL, cudaStream_t sH)
     cudaEvent_t evCentre = e->capturing ? e->cCentre : e->evCentre;
     bool recentre = false;
     for (ibl_lb *lb : e->m) recentre = recentre || lb->v.recentre != 0;
-    cudaError_t err = iblb::launch_ensemble_pre(e->v, step, sH, e->hi_prio);
+    cudaError_t err = iblb::launch_ensemble_tri(e->v, step, sH, e->hi_prio);
     if (err == cudaSuccess && recentre) err = cudaEventRecord(evCentre, sH);
+    if (err == cudaSuccess) err = iblb::launch_ensemble_spread(e->v, step, sH, e->hi_prio);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(sH, evFar[par ^ 1], 0);
     if (err == cudaSuccess) err = iblb::launch_ensemble_near(e->v, step, sH, e->hi_prio);
     if (err == cudaSuccess) err = cudaEventRecord(evNear[par], sH);

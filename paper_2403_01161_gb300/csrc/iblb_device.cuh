@@ -339,9 +339,8 @@ __device__ __forceinline__ bool node_in_patch(const LbView &L, const Ctl *c, int
 // |N|), N its normal.  FP64 mesh geometry for either population precision.
 // tri_moment evaluates m once per triangle for the ensemble's force kernel.
 template <class P>
-__device__ __forceinline__ void tri_moment(const MeshView &M, const int t, double m[3], const P &K)
+__device__ __forceinline__ void tri_moment(const MeshView &M, const int t, double m[3], double (&x)[3][3], const P &K)
 {
-    double x[3][3];
     for (int k = 0; k < 3; ++k) {
         const int v = K.ld(M.tris + 3 * t + k);
         for (int a = 0; a < 3; ++a) x[k][a] = K.ld(M.r + 3 * v + a);
@@ -354,6 +353,22 @@ __device__ __forceinline__ void tri_moment(const MeshView &M, const int t, doubl
     cross3(e1, e2, N);
     const double s = -0.5 * M.sigma * rsqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
     for (int a = 0; a < 3; ++a) m[a] = s * N[a];
+}
+
+// Sums of four values over a group of LANES lanes: the lane's result is the
+// sum of value lane / (LANES / 4).  Halving the values with the lanes takes
+// 2 + 1 + log2(LANES) - 2 additions instead of 4 log2(LANES).
+template <int LANES>
+__device__ __forceinline__ double group_sum4(const double (&v)[4])
+{
+    static_assert(LANES >= 4, "a lane per value");
+    const bool hi = (threadIdx.x & (LANES / 2)) != 0, mid = (threadIdx.x & (LANES / 4)) != 0;
+    const double a0 = __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], LANES / 2);
+    const double a1 = __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], LANES / 2);
+    const double b0 = (hi ? v[2] : v[0]) + a0, b1 = (hi ? v[3] : v[1]) + a1;
+    double c = (mid ? b1 : b0) + __shfl_xor_sync(0xffffffffu, mid ? b0 : b1, LANES / 4);
+    for (int o = LANES / 8; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    return c;
 }
 
 // ---------------------------------------------------------------------------

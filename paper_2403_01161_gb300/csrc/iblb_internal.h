@@ -97,8 +97,7 @@ struct MeshView {
     double *s0, *s1, *s2;  // regularisation scratch, [nv][3] each
     double *tm;            // [nt][3] m_t = -sigma N_t / (2 |N_t|) at the current positions (ensemble: written by the batched triangle kernel, read by the batched force kernel)
     double *part;          // per-block bounding-box partials of the interpolation kernel, [blocks][6]
-    double *cpart;         // re-centring: per-block volume and first moment, [kCentreBlocks][4]
-    double *obs_part;      // per-block partial sums of the shape-record kernel, [kObsBlocksMax][11]
+    double *obs_part;      // per-block partial sums of the shape-record kernel, [kObsBlocksMax][11], and of the re-centring
     ibl_observables *ring;
     int ring_cap;
     // Adjoint recording (null otherwise): the force/spread kernel of a step
@@ -188,6 +187,8 @@ constexpr int kStagedShapes = 2;
 cudaError_t launch_near(const LbView &L, bool odd, bool record, int pbuf, cudaStream_t s, int prio = 0);
 enum { LAUNCH_FULL = 0, LAUNCH_FAR = 1 };
 cudaError_t launch_convert_frames(const LbView &L, int k0, int k1, cudaStream_t s);
+// forces + spread, the patch of the next step (buffer next_buf), and where the
+// lattice view asks for them the step's centre of mass and inside flags
 cudaError_t launch_spread(const LbView &L, const MeshView &M, int next_buf, cudaStream_t s, int prio = 0);
 cudaError_t launch_interp(const LbView &L, const MeshView &M, cudaStream_t s, int prio = 0);
 // Lanes per mesh node in the forward force/spread and interpolation kernels
@@ -197,11 +198,6 @@ cudaError_t launch_interp(const LbView &L, const MeshView &M, cudaStream_t s, in
 constexpr int kFwdLanes = 8;
 static_assert(kFwdLanes == 4 || kFwdLanes == 8 || kFwdLanes == 16, "lanes per mesh node");
 constexpr int kFwdNodesPerBlock = 128 / kFwdLanes;
-// re-centring: the droplet's centre of mass at the current positions into ctl->centre[buf]
-constexpr int kCentreBlocks = 16;
-cudaError_t launch_centre(const LbView &L, const MeshView &M, int buf, cudaStream_t s, int prio = 0);
-// viscosity ratio: the inside flags of the patch nodes of step `buf` from the current positions
-cudaError_t launch_indicator(const LbView &L, const MeshView &M, int buf, cudaStream_t s, int prio = 0);
 cudaError_t launch_regularize(const LbView &L, const MeshView &M, const RegParams &p, int buf, cudaStream_t s,
                               int prio = 0);
 // the members with due[k] != 0, one launch per group
@@ -210,12 +206,13 @@ cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<c
 cudaError_t launch_observables(const LbView &L, const MeshView &M, cudaStream_t s, int prio = 0);
 cudaError_t launch_patch_from_mesh(const LbView &L, const MeshView &M, int buf, cudaStream_t s);
 // Ensemble step phases (two streams, as the single droplet's step):
-// helper stream: pre (centre, triangle moments, forces + spread of the next
-// patch) then near (patch nodes, after the previous far update) then interp;
+// helper stream: tri (triangle moments, centres), spread (forces + spread, the
+// next patch) then near (patch nodes, after the previous far update) then interp;
 // bound stream: far (nodes outside each member's patch, closes each
 // member's step, after the previous near update).
 constexpr int kEnsNearBlocks = 48;  // blocks per member of the batched patch-node kernel
-cudaError_t launch_ensemble_pre(const EnsembleView &E, long long step, cudaStream_t s, int prio);
+cudaError_t launch_ensemble_tri(const EnsembleView &E, long long step, cudaStream_t s, int prio);
+cudaError_t launch_ensemble_spread(const EnsembleView &E, long long step, cudaStream_t s, int prio);
 cudaError_t launch_ensemble_near(const EnsembleView &E, long long step, cudaStream_t s, int prio);
 cudaError_t launch_ensemble_far(const EnsembleView &E, long long step, cudaStream_t s);
 cudaError_t launch_ensemble_interp(const EnsembleView &E, cudaStream_t s, int prio);

@@ -892,21 +892,21 @@ __device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, 
     const bool valid = gid < M.nv;
     const int i = valid ? gid : M.nv - 1;
     const P K;
-    double F[3] = {0.0, 0.0, 0.0};
     const int k0 = K.ld(M.n2t_ptr + i), k1 = K.ld(M.n2t_ptr + i + 1);
     double ra;
     const NodeStencil<T> S = node_stencil<T, LANES, false>(L, M.r + 3 * i, lane, K, ra);
     double xi[3];
     if constexpr (!STORED)
         for (int a = 0; a < 3; ++a) xi[a] = K.ld(M.r + 3 * i + a);
-    for (int k = k0 + lane; k < k1; k += LANES) {
+    // force of the incidence k: triangle t with the node in position `slot`
+    auto term = [&](const int k, double (&g)[3]) {
         const int e = K.ld(M.n2t + k);
         const int t = e / 3, slot = e - 3 * t;
         const int vp = K.ld(M.tris + (slot == 2 ? e - 2 : e + 1)), vq = K.ld(M.tris + (slot == 0 ? e + 2 : e - 1));
         double p[3], q[3];
         for (int a = 0; a < 3; ++a) p[a] = K.ld(M.r + 3 * vp + a);
         for (int a = 0; a < 3; ++a) q[a] = K.ld(M.r + 3 * vq + a);
-        double m[3], g[3];
+        double m[3];
         if constexpr (STORED) {
             for (int a = 0; a < 3; ++a) m[a] = K.ld(M.tm + 3 * t + a);
         } else {
@@ -919,19 +919,31 @@ __device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, 
         }
         const double dd[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
         cross3(m, dd, g);
+    };
+    double F[4] = {0.0, 0.0, 0.0, 0.0};
+    int k = k0 + lane;
+    if (k < k1) {
+        double g[3];
+        term(k, g);
+        for (int a = 0; a < 3; ++a) F[a] = g[a];
+    }
+    while ((k += LANES) < k1) {  // valences above LANES
+        double g[3];
+        term(k, g);
         for (int a = 0; a < 3; ++a) F[a] += g[a];
     }
-    for (int o = LANES / 2; o > 0; o >>= 1)
-        for (int a = 0; a < 3; ++a) F[a] += __shfl_xor_sync(0xffffffffu, F[a], o, LANES);
-    if (valid && lane < 3) {
-        M.fn[3 * i + lane] = lane == 0 ? F[0] : (lane == 1 ? F[1] : F[2]);
-        if (M.rec_r) M.rec_r[3 * i + lane] = ra;
-    }
+    const double Fa = group_sum4<LANES>(F);  // component lane / (LANES / 4)
+    const int comp = lane / (LANES / 4);
+    if (valid && lane % (LANES / 4) == 0 && comp < 3) M.fn[3 * i + comp] = Fa;
+    if (M.rec_r && valid && lane < 3) M.rec_r[3 * i + lane] = ra;
+    const int w0 = (threadIdx.x & 31) & ~(LANES - 1);
+    const T Ft = T(Fa);
+    const T Fx = __shfl_sync(0xffffffffu, Ft, w0), Fy = __shfl_sync(0xffffffffu, Ft, w0 + LANES / 4),
+            Fz = __shfl_sync(0xffffffffu, Ft, w0 + LANES / 2);
     if (valid && !S.ok && lane == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_WALL);
     if (!valid || !S.ok) return;
     const int nx = L.n[0], nxy = L.n[0] * L.n[1];
     T *force = static_cast<T *>(L.force);  // [nodes][4]
-    const T Fx = T(F[0]), Fy = T(F[1]), Fz = T(F[2]);
     T w[4];
     int x[4];
 #pragma unroll
@@ -944,8 +956,8 @@ __device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, 
     const T wy = stencil_w(S.f[1], S.s[1], b);
     const int y = stencil_at(S.base[1], b, L.n[1]) * nx;
 #pragma unroll
-    for (int k = 0; k < 16 / LANES; ++k) {
-        const int c = (lane >> 2) + (LANES / 4) * k;
+    for (int j = 0; j < 16 / LANES; ++j) {
+        const int c = (lane >> 2) + (LANES / 4) * j;
         const T wz = stencil_w(S.f[2], S.s[2], c);
         const int row = y + stencil_at(S.base[2], c, L.n[2]) * nxy;
 #pragma unroll
@@ -956,83 +968,106 @@ __device__ __forceinline__ void spread_body(const LbView &L, const MeshView &M, 
     }
 }
 
-// Ensemble: m_t of every triangle of every member at the current positions
-// (Eq. (pi_drop)), once per step, for the batched force kernel that follows
-// on the same stream; blockIdx.y is the member within the group.
-template <class P>
-__global__ void __launch_bounds__(128) k_tri_moment_batched(const __grid_constant__ MeshGroup MG)
-{
-    const MeshView &M = MG.v[blockIdx.y];
-    const P K;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < M.nt; t += gridDim.x * blockDim.x) {
-        double m[3];
-        tri_moment(M, t, m, K);
-        for (int a = 0; a < 3; ++a) K.st(M.tm + 3 * t + a, m[a]);
-    }
-}
-
-template <typename T, int LANES>
-__global__ void __launch_bounds__(128) k_spread(LbView L, MeshView M, int next_buf, int nblk)
-{
-    // the first block reduces the patch; node groups are block-strided over the others
-    if (blockIdx.x == 0) {
-        patch_from_rows<L2Keep>(L, M, next_buf);
-        return;
-    }
-    for (int b = (int)blockIdx.x - 1; b < nblk; b += (int)gridDim.x - 1) spread_body<T, false, LANES>(L, M, b);
-}
-
 // Re-centring (Sec. 3.2: the linearisation is centred on the droplet's
-// centre of mass).  kCentreBlocks blocks per droplet sum the volume V and
-// first moment m of the region the mesh encloses over the signed tetrahedra
-// (box centre, a, b, c) of the triangles, block b taking triangles b, b +
-// kCentreBlocks, ... thread by thread.  Each block writes its sums to
-// M.cpart; the last block to finish adds the rows in block order
-// (deterministic) and stores the step's centre, box centre + m / V, in
-// buffer `buf`.  Runs after the interpolation of the previous step and
-// before any lattice update of this step.
-constexpr int kCentreThreads = 128;
+// centre of mass).  `nblk` blocks per droplet sum six times the volume V and
+// twenty-four times its first moment m over the signed tetrahedra (box centre,
+// a, b, c) of the triangles.  Each block writes its sums to a row of M.obs_part
+// (the shape record, its other user, runs on the same stream); the last block
+// to finish adds the rows in a fixed order and stores the step's centre, box
+// centre + m / V, in buffer `buf`.  Runs after the interpolation of the
+// previous step and before any lattice update of this step.
+constexpr int kCentreBlocksMax = 128;
+static_assert(kCentreBlocksMax <= kObsBlocksMax, "rows of obs_part");
 
-__device__ __forceinline__ void centre_of_mass(const LbView &L, const MeshView &M, const int blk, const int buf)
+// A triangle's share: 6 V and 24 m about the box centre.
+__device__ __forceinline__ void centre_term(const double (&p)[3][3], double (&v)[4])
 {
-    __shared__ double sh[kCentreThreads / 32][4];
+    double bc[3];
+    cross3(p[1], p[2], bc);
+    const double vt = p[0][0] * bc[0] + p[0][1] * bc[1] + p[0][2] * bc[2];
+    v[0] += vt;
+    for (int a = 0; a < 3; ++a) v[1 + a] += vt * (p[0][a] + p[1][a] + p[2][a]);
+}
+__device__ __forceinline__ void centre_ref(const LbView &L, double (&ref)[3])
+{
+    for (int a = 0; a < 3; ++a) ref[a] = 0.5 * (L.n[a] - 1);
+}
+__device__ __forceinline__ void centre_finish(const LbView &L, const MeshView &M, const double (&v)[4], const int blk,
+                                              const int nblk, const int buf)
+{
+    __shared__ double sh[kIbThreads / 32][4];
     __shared__ int last;
-    const double ref[3] = {0.5 * (L.n[0] - 1), 0.5 * (L.n[1] - 1), 0.5 * (L.n[2] - 1)};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double w[4] = {v[0], v[1], v[2], v[3]};
+    const double s = group_sum4<32>(w);
+    if ((lane & 7) == 0) sh[warp][lane >> 3] = s;
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double t = sh[0][threadIdx.x];
+        for (int k = 1; k < kIbThreads / 32; ++k) t += sh[k][threadIdx.x];
+        M.obs_part[4 * blk + threadIdx.x] = t;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&L.ctl->cen_ticket, 1u) == (unsigned)(nblk - 1) ? 1 : 0;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // warp 0: lane sums component lane / 8 of every eighth row
+    if (warp == 0) {
+        double t = 0.0;
+        for (int b = lane & 7; b < nblk; b += 8) t += __ldcg(M.obs_part + 4 * b + (lane >> 3));
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        const double V = __shfl_sync(0xffffffffu, t, 0);
+        if ((lane & 7) == 0 && lane > 0) {
+            const int a = (lane >> 3) - 1;
+            L.ctl->centre[buf][a] = 0.5 * ((a == 0 ? L.n[0] : (a == 1 ? L.n[1] : L.n[2])) - 1) + t / (4.0 * V);
+        }
+        if (lane == 0) L.ctl->cen_ticket = 0u;
+    }
+}
+__device__ __forceinline__ void centre_unit(const LbView &L, const MeshView &M, const int blk, const int nblk,
+                                            const int buf)
+{
     const L2Keep K;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int t = blk * kCentreThreads + (int)threadIdx.x; t < M.nt; t += kCentreBlocks * kCentreThreads) {
+    double ref[3], v[4] = {0.0, 0.0, 0.0, 0.0};
+    centre_ref(L, ref);
+    for (int t = blk * kIbThreads + (int)threadIdx.x; t < M.nt; t += nblk * kIbThreads) {
         double p[3][3];
         for (int c = 0; c < 3; ++c) {
             const int q = K.ld(M.tris + 3 * t + c);
             for (int a = 0; a < 3; ++a) p[c][a] = K.ld(M.r + 3 * q + a) - ref[a];
         }
-        double bc[3];
-        cross3(p[1], p[2], bc);
-        const double vt = (p[0][0] * bc[0] + p[0][1] * bc[1] + p[0][2] * bc[2]) / 6.0;
-        v[0] += vt;
-        for (int a = 0; a < 3; ++a) v[1 + a] += vt * (p[0][a] + p[1][a] + p[2][a]) / 4.0;
+        centre_term(p, v);
     }
-    block_sum<4>(v, sh);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 4; ++k) M.cpart[4 * blk + k] = v[k];
-        __threadfence();
-        last = atomicAdd(&L.ctl->cen_ticket, 1u) == (unsigned)(kCentreBlocks - 1) ? 1 : 0;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (threadIdx.x == 0) {
-        double w[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int b = 0; b < kCentreBlocks; ++b)
-            for (int k = 0; k < 4; ++k) w[k] += __ldcg(M.cpart + 4 * b + k);
-        for (int a = 0; a < 3; ++a) L.ctl->centre[buf][a] = ref[a] + w[1 + a] / w[0];
-        L.ctl->cen_ticket = 0u;
-    }
+    centre_finish(L, M, v, blk, nblk, buf);
 }
 
-__global__ void __launch_bounds__(kCentreThreads) k_centre(LbView L, MeshView M, int buf)
+// Ensemble: m_t of every triangle of every member at the current positions
+// (Eq. (pi_drop)), once per step, for the batched force kernel that follows
+// on the same stream, and with re-centring the centre of mass from the same
+// positions; blockIdx.y is the member within the group.
+template <class P>
+__global__ void __launch_bounds__(128)
+    k_tri_moment_batched(const __grid_constant__ LbGroup LG, const __grid_constant__ MeshGroup MG, const int buf)
 {
-    centre_of_mass(L, M, blockIdx.x, buf);
+    const LbView &L = LG.v[blockIdx.y];
+    const MeshView &M = MG.v[blockIdx.y];
+    const P K;
+    const bool centre = L.recentre != 0;
+    double ref[3], v[4] = {0.0, 0.0, 0.0, 0.0};
+    if (centre) centre_ref(L, ref);
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < M.nt; t += gridDim.x * blockDim.x) {
+        double x[3][3], m[3];
+        tri_moment(M, t, m, x, K);
+        for (int a = 0; a < 3; ++a) K.st(M.tm + 3 * t + a, m[a]);
+        if (centre) {
+            for (int c = 0; c < 3; ++c)
+                for (int a = 0; a < 3; ++a) x[c][a] -= ref[a];
+            centre_term(x, v);
+        }
+    }
+    if (centre) centre_finish(L, M, v, blockIdx.x, gridDim.x, buf);
 }
 
 // Viscosity ratio (Sec. 2: droplet viscosity chi mu): the inside flags of the
@@ -1054,9 +1089,9 @@ __device__ __forceinline__ double edge_fn(double ax, double ay, double bx, doubl
     return __dsub_rn(__dmul_rn(__dsub_rn(bx, ax), __dsub_rn(qy, ay)), __dmul_rn(__dsub_rn(by, ay), __dsub_rn(qx, ax)));
 }
 
-__global__ void __launch_bounds__(128) k_indicator(LbView L, MeshView M, int buf)
+__device__ __forceinline__ void indicator_unit(const LbView &L, const MeshView &M, const int blk, const int buf)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blk * kIbThreads + (int)threadIdx.x;
     if (t >= M.nt) return;
     const Ctl *c = L.ctl;
     if (c->patch_ext[buf][0] < 0 || c->patch_ext[buf][1] < 0 || c->patch_ext[buf][2] < 0) return;
@@ -1093,11 +1128,34 @@ __global__ void __launch_bounds__(128) k_indicator(LbView L, MeshView M, int buf
         }
 }
 
-// Ensemble version: blockIdx.y is the member within the group.
-__global__ void __launch_bounds__(kCentreThreads)
-    k_centre_batched(const __grid_constant__ LbGroup LG, const __grid_constant__ MeshGroup MG, int buf)
+// Blocks of one launch: the patch of the next step (block 0), then, where the
+// step needs them, nc blocks for its centre of mass and ni for its inside
+// flags, then the node groups.  All of them only read the positions, so none
+// waits for another: as launches of their own, centre and flags put 16 and 10
+// us (cold) ahead of the forces on the droplet chain.
+template <typename T, int LANES, bool EXTRA>
+__global__ void __launch_bounds__(128) k_spread(LbView L, MeshView M, int next_buf, int nc, int ni)
 {
-    centre_of_mass(LG.v[blockIdx.y], MG.v[blockIdx.y], blockIdx.x, buf);
+    int b = (int)blockIdx.x;
+    if (b == 0) {
+        patch_from_rows<L2Keep>(L, M, next_buf);
+        return;
+    }
+    b -= 1;
+    if constexpr (EXTRA) {
+        const int buf = next_buf == 0 ? 2 : next_buf - 1;  // this step's
+        if (b < nc) {
+            centre_unit(L, M, b, nc, buf);
+            return;
+        }
+        b -= nc;
+        if (b < ni) {
+            indicator_unit(L, M, b, buf);
+            return;
+        }
+        b -= ni;
+    }
+    spread_body<T, false, LANES>(L, M, b);
 }
 
 template <typename T, int LANES, class P = L2Keep>
@@ -1561,42 +1619,30 @@ static int fwd_lanes(const MeshView &M)
     return (long long)M.nv * 16 <= (long long)sm_count() * kIbThreads ? 16 : kFwdLanes;
 }
 
-// Blocks of the single droplet's node-group kernels: one per group of
-// nodes.  (The kernels are block-strided, so a grid may be capped; capped at
-// two blocks per SM, the 256^3 step took 431 instead of 437 us and the 200^3
-// step without regularisation 218.6 instead of 223.0 us, but the 200^3 step
-// regularised after every step 254 instead of 235 us: the longer droplet
-// chain then no longer fits beside the outside update.)
-static unsigned ib_grid(int nblk) { return (unsigned)nblk; }
+template <typename T, int LANES>
+static cudaError_t spread_t(const LbView &L, const MeshView &M, int next_buf, cudaStream_t s, int prio)
+{
+    const int nblk = (int)blocks_for((long long)M.nv * LANES, kIbThreads), nt = (int)blocks_for(M.nt, kIbThreads);
+    const int nc = L.recentre ? (nt < kCentreBlocksMax ? nt : kCentreBlocksMax) : 0, ni = L.visc ? nt : 0;
+    const dim3 g(1 + nc + ni + nblk), b(kIbThreads);
+    if (nc + ni > 0) return launch_p(k_spread<T, LANES, true>, g, b, s, prio, L, M, next_buf, nc, ni);
+    return launch_p(k_spread<T, LANES, false>, g, b, s, prio, L, M, next_buf, 0, 0);
+}
 
 cudaError_t launch_spread(const LbView &L, const MeshView &M, int next_buf, cudaStream_t s, int prio)
 {
-    const int lanes = fwd_lanes(M);
-    const int nblk = (int)blocks_for((long long)M.nv * lanes, kIbThreads);
-    const dim3 g(1 + ib_grid(nblk)), b(kIbThreads);  // and the patch block
-    if (lanes == 16) {
-        if (L.precision == IBL_FP64) return launch_p(k_spread<double, 16>, g, b, s, prio, L, M, next_buf, nblk);
-        return launch_p(k_spread<float, 16>, g, b, s, prio, L, M, next_buf, nblk);
-    }
-    if (L.precision == IBL_FP64) return launch_p(k_spread<double, kFwdLanes>, g, b, s, prio, L, M, next_buf, nblk);
-    return launch_p(k_spread<float, kFwdLanes>, g, b, s, prio, L, M, next_buf, nblk);
-}
-
-cudaError_t launch_centre(const LbView &L, const MeshView &M, int buf, cudaStream_t s, int prio)
-{
-    return launch_p(k_centre, dim3(kCentreBlocks), dim3(kCentreThreads), s, prio, L, M, buf);
-}
-
-cudaError_t launch_indicator(const LbView &L, const MeshView &M, int buf, cudaStream_t s, int prio)
-{
-    return launch_p(k_indicator, dim3(blocks_for(M.nt, 128)), dim3(128), s, prio, L, M, buf);
+    if (fwd_lanes(M) == 16)
+        return L.precision == IBL_FP64 ? spread_t<double, 16>(L, M, next_buf, s, prio)
+                                       : spread_t<float, 16>(L, M, next_buf, s, prio);
+    return L.precision == IBL_FP64 ? spread_t<double, kFwdLanes>(L, M, next_buf, s, prio)
+                                   : spread_t<float, kFwdLanes>(L, M, next_buf, s, prio);
 }
 
 cudaError_t launch_interp(const LbView &L, const MeshView &M, cudaStream_t s, int prio)
 {
     const int lanes = fwd_lanes(M);
     const int nblk = (int)blocks_for((long long)M.nv * lanes, kIbThreads);
-    const dim3 g(ib_grid(nblk)), b(kIbThreads);
+    const dim3 g(nblk), b(kIbThreads);
     if (lanes == 16) {
         if (L.precision == IBL_FP64) return launch_p(k_interp<double, 16>, g, b, s, prio, L, M, nblk);
         return launch_p(k_interp<float, 16>, g, b, s, prio, L, M, nblk);
@@ -1653,48 +1699,53 @@ static int chain_grid(const EnsembleView &E, int nb)
     return nb < cap ? nb : cap;
 }
 
-template <class P>
-static cudaError_t ensemble_pre_t(const EnsembleView &E, int m0, int m1, int pbuf, int nxt, cudaStream_t s, int prio)
+cudaError_t launch_ensemble_tri(const EnsembleView &E, long long step, cudaStream_t s, int prio)
 {
+    const int pbuf = (int)(step % 3), n = (int)E.lv.size();
+    const bool keep = ens_shape_keep(ens_shape(E));
     Groups &G = groups();
-    bool recentre = false;
-    int nt_max = 0;
-    for (int k = m0; k < m1; ++k) {
-        recentre = recentre || E.lv[k].recentre != 0;
-        nt_max = E.mv[k].nt > nt_max ? E.mv[k].nt : nt_max;
+    for (int m0 = 0; m0 < n; m0 += kGroup) {
+        const int m1 = m0 + kGroup < n ? m0 + kGroup : n;
+        fill_group(E, m0, m1);
+        int nt_max = 0;
+        for (int k = m0; k < m1; ++k) nt_max = E.mv[k].nt > nt_max ? E.mv[k].nt : nt_max;
+        int tb = (nt_max + 127) / 128;
+        if (ens_shape_capped(ens_shape(E))) {
+            const int cap = ens_shape_cap(ens_shape(E)) * sm_count() / (m1 - m0);
+            tb = tb < cap ? tb : (cap < 1 ? 1 : cap);
+        }
+        tb = tb < kCentreBlocksMax ? tb : kCentreBlocksMax;
+        const dim3 g(tb, m1 - m0), b(kIbThreads);
+        const cudaError_t e = keep ? launch_p(k_tri_moment_batched<L2Keep>, g, b, s, prio, G.lg, G.mg, pbuf)
+                                   : launch_p(k_tri_moment_batched<L2Plain>, g, b, s, prio, G.lg, G.mg, pbuf);
+        if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaSuccess;
-    if (recentre)
-        e = launch_p(k_centre_batched, dim3(kCentreBlocks, m1 - m0), dim3(kCentreThreads), s, prio, G.lg, G.mg, pbuf);
-    int tb = (nt_max + 127) / 128;
-    if (ens_shape_capped(ens_shape(E))) {
-        const int cap = ens_shape_cap(ens_shape(E)) * sm_count() / (m1 - m0);
-        tb = tb < cap ? tb : (cap < 1 ? 1 : cap);
-    }
-    if (e == cudaSuccess) e = launch_p(k_tri_moment_batched<P>, dim3(tb, m1 - m0), dim3(128), s, prio, G.mg);
-    const int nb0 = E.node_start[m0], nb = E.node_start[m1] - nb0;
-    const dim3 g(chain_grid(E, nb + m1 - m0));
-    if (e == cudaSuccess) {
-        if (E.precision == IBL_FP64)
-            e = launch_p(k_spread_batched<double, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, m1 - m0, nb0, nb,
-                         E.node_member, E.node_start_d, nxt);
-        else
-            e = launch_p(k_spread_batched<float, P>, g, dim3(kIbThreads), s, prio, G.lg, G.mg, m0, m1 - m0, nb0, nb,
-                         E.node_member, E.node_start_d, nxt);
-    }
-    return e;
+    return cudaSuccess;
 }
 
-cudaError_t launch_ensemble_pre(const EnsembleView &E, long long step, cudaStream_t s, int prio)
+template <typename T, class P>
+static cudaError_t ensemble_spread_t(const EnsembleView &E, int m0, int m1, int nxt, cudaStream_t s, int prio)
 {
-    const int pbuf = (int)(step % 3), nxt = (int)((step + 1) % 3);
-    const int n = (int)E.lv.size();
+    Groups &G = groups();
+    const int nb0 = E.node_start[m0], nb = E.node_start[m1] - nb0;
+    return launch_p(k_spread_batched<T, P>, dim3(chain_grid(E, nb + m1 - m0)), dim3(kIbThreads), s, prio, G.lg, G.mg, m0,
+                    m1 - m0, nb0, nb, E.node_member, E.node_start_d, nxt);
+}
+
+cudaError_t launch_ensemble_spread(const EnsembleView &E, long long step, cudaStream_t s, int prio)
+{
+    const int nxt = (int)((step + 1) % 3), n = (int)E.lv.size();
     const bool keep = ens_shape_keep(ens_shape(E));
     for (int m0 = 0; m0 < n; m0 += kGroup) {
         const int m1 = m0 + kGroup < n ? m0 + kGroup : n;
         fill_group(E, m0, m1);
-        const cudaError_t e = keep ? ensemble_pre_t<L2Keep>(E, m0, m1, pbuf, nxt, s, prio)
-                                   : ensemble_pre_t<L2Plain>(E, m0, m1, pbuf, nxt, s, prio);
+        cudaError_t e;
+        if (E.precision == IBL_FP64)
+            e = keep ? ensemble_spread_t<double, L2Keep>(E, m0, m1, nxt, s, prio)
+                     : ensemble_spread_t<double, L2Plain>(E, m0, m1, nxt, s, prio);
+        else
+            e = keep ? ensemble_spread_t<float, L2Keep>(E, m0, m1, nxt, s, prio)
+                     : ensemble_spread_t<float, L2Plain>(E, m0, m1, nxt, s, prio);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
