@@ -830,12 +830,12 @@ struct EnsembleLayout {
     int lat_blocks[2] = {0, 0}, node_blocks = 0;
 };
 
-// Blocks of the batched lattice update of one member with nt threads per
-// block: whole blocks per z plane.
-long long lattice_blocks(const ibl_lb *lb, int nt)
+// Blocks of the batched lattice update of one member with nt threads and
+// `tiles` tiles per block.
+long long lattice_blocks(const ibl_lb *lb, int nt, int tiles)
 {
-    const long long nxy = (long long)lb->v.n[0] * lb->v.n[1];
-    return (nxy + nt - 1) / nt * lb->v.n[2];
+    const long long per = (long long)nt * tiles;
+    return ((long long)lb->v.nodes + per - 1) / per;
 }
 
 int ensemble_layout(int n, ibl_lb *const *members, EnsembleLayout &L, std::string &why)
@@ -855,8 +855,9 @@ int ensemble_layout(int n, ibl_lb *const *members, EnsembleLayout &L, std::strin
             why = "an ensemble member's z plane exceeds 2^22 nodes";
             return IBL_EINVAL;
         }
-        lat[0] += lattice_blocks(lb, 128);
-        lat[1] += lattice_blocks(lb, 256);
+        // the tables are sized for one tile per block, the most blocks there are
+        lat[0] += lattice_blocks(lb, 128, 1);
+        lat[1] += lattice_blocks(lb, 256, 1);
         node += ((long long)lb->mesh->v.nv + iblb::kFwdNodesPerBlock - 1) / iblb::kFwdNodesPerBlock;
     }
     if (lat[0] > 0x7fffffffLL) {
@@ -1177,7 +1178,6 @@ int ibl_lb_create(const ibl_lb_params *p, const double *A_frames, int n_frames, 
     v.rule = p->edge_rule;
     v.omega = 1.0 / p->tau;
     v.omega_f = (float)(1.0 / p->tau);
-    v.inv_nx = 1.0f / (float)p->n[0];
     v.div_nx = iblb::div_by_const(p->n[0]);
     v.div_nxy = iblb::div_by_const(p->n[0] * p->n[1]);
     v.f = lb->ws + L.f;
@@ -1883,6 +1883,9 @@ int ibl_ensemble_create(int n, ibl_lb *const *members, void *workspace, size_t b
     if (!workspace || bytes < L.total) return fail(IBL_ENOMEM, "ensemble workspace too small");
     if (((uintptr_t)workspace & 255) != 0) return fail(IBL_EINVAL, "workspace must be 256-byte aligned");
     const ibl_lb *m0 = members[0];
+    bool recentre = false;
+    for (int k = 0; k < n; ++k) recentre = recentre || members[k]->v.recentre != 0;
+    const int tiles = recentre ? iblb::kEnsTilesCentred : iblb::kEnsTiles;
     std::vector<LbView> lv;
     std::vector<MeshView> mv;
     std::vector<int> lat_member[2], lat_start[2], node_member, node_start;
@@ -1898,7 +1901,7 @@ int ibl_ensemble_create(int n, ibl_lb *const *members, void *workspace, size_t b
         mv.push_back(lb->mesh->v);
         for (int t = 0; t < 2; ++t) {
             lat_start[t].push_back((int)lat_member[t].size());
-            for (long long b = 0; b < lattice_blocks(lb, t == 0 ? 128 : 256); ++b) lat_member[t].push_back(k);
+            for (long long b = 0; b < lattice_blocks(lb, t == 0 ? 128 : 256, tiles); ++b) lat_member[t].push_back(k);
         }
         node_start.push_back((int)node_member.size());
         for (int b = 0; b < (lb->mesh->v.nv + iblb::kFwdNodesPerBlock - 1) / iblb::kFwdNodesPerBlock; ++b)
@@ -1936,6 +1939,7 @@ int ibl_ensemble_create(int n, ibl_lb *const *members, void *workspace, size_t b
     v.node_start = node_start;
     v.precision = m0->p.precision;
     v.shape = iblb::kEnsDefaultShape;
+    v.recentre = recentre;
     *out = en;
     return IBL_OK;
 }

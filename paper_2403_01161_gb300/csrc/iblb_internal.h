@@ -63,8 +63,7 @@ struct LbView {
     int rule;           // IBL_EDGE_*
     double omega;       // 1 / tau
     float omega_f;
-    DivBy div_nx, div_nxy;  // node -> row and z plane in the single-lattice kernel
-    float inv_nx;       // 1 / n[0] (rounded): row of a node within its z plane in the batched lattice kernel
+    DivBy div_nx, div_nxy;  // node -> row and z plane
     void *f;            // [19][qs]
     void *force;        // [nodes][4]: x, y, z, 0 (one 16-byte record per node in FP32)
     void *vel;          // [nodes][4]
@@ -129,8 +128,8 @@ struct MeshGroup {
 // Launch shapes of the ensemble step, the candidates of ibl_ensemble_tune:
 // shape k = 8 c + 4 p + 2 t + w takes w resident waves of blocks of L2
 // prefetch distance and 128 (t = 0) or 256 (t = 1) threads per block in the
-// batched lattice update (each block takes that many consecutive nodes of
-// one z plane of one member); p = 0 keeps the droplet-side working set in
+// batched lattice update (a block takes kEnsTiles runs of that many consecutive
+// nodes of one member); p = 0 keeps the droplet-side working set in
 // L2 (evict_last, as the single droplet does), p = 1 uses the default
 // policy; c = 1, 2, 3 caps the grids of the droplet-side kernels at 1, 2, 4
 // blocks per SM (they then stride over their work), c = 0 launches one
@@ -142,6 +141,9 @@ constexpr bool ens_shape_keep(int k) { return (k & 4) == 0; }
 constexpr int ens_shape_cap(int k) { return (k >> 3) == 0 ? 0 : ((k >> 3) == 3 ? 4 : (k >> 3)); }
 constexpr bool ens_shape_capped(int k) { return ens_shape_cap(k) > 0; }
 constexpr int kEnsDefaultShape = 16;
+// Tiles of consecutive nodes per block of the batched lattice update (see
+// k_lattice_batched).
+constexpr int kEnsTiles = 4, kEnsTilesCentred = 1;
 
 struct EnsembleView {
     std::vector<LbView> lv;      // host copies of the member views
@@ -155,6 +157,7 @@ struct EnsembleView {
     std::vector<int> node_start;
     int precision;
     int shape;                   // kEnsShapes index of the batched lattice launch
+    bool recentre;               // some member is re-centred (its batched lattice launch: kEnsTilesCentred tiles per block)
 };
 
 // Discrete adjoint of one step (device pointers in the adjoint workspace).

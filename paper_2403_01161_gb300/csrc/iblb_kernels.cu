@@ -752,51 +752,57 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lattice_near(Lb
 // the lattices of a group of members (the patches are updated concurrently
 // by k_lattice_near_batched on the helper stream).  Block b works for member
 // blk_member[b0 + b] (view G.v[member - m0], read from the kernel
-// parameters) as its local block l = b0 + b - blk_start[member]: NT
-// consecutive nodes of z plane l / bpp (bpp = blocks per plane) in x-fastest
-// order, starting at node (l mod bpp) NT of the plane; the row of a node is
-// p / n_x, taken as floor((p + 1/2) inv_nx), exact while n_x n_y < 2^22 (the
-// fraction of (p + 1/2)/n_x stays 1/(2 n_x) away from an integer, more than
-// the float rounding).  The first thread of a member's first block closes
-// that member's step, as the single-droplet far kernel does.  Each thread
-// prefetches into L2 its (x, y) `ahead` planes further (about `waves`
-// resident waves of blocks later).
+// parameters) as its local block l = b0 + b - blk_start[member]: `tiles`
+// tiles of NT consecutive nodes of the flattened box, from node l tiles NT
+// on.  The first thread of a member's first block closes that member's step,
+// as the single-droplet far kernel does.  With prefetch each thread fetches
+// into L2 the node `ahead_nodes` further.
+// Several tiles per block because a block starts with a chain of its own, the
+// member from the table and then its view from the parameters (64 views do not
+// stay in the constant cache), before its first population load: four tiles
+// took the step of 32 droplets from 508 to 470 us (two 489, eight 474).  Where
+// a member is re-centred (CEN, for the whole ensemble) the droplet chain is as
+// long as the outside update, and its blocks wait for the outside update's to
+// end: there one tile is faster (16 regularised, centred droplets 232 against
+// 239 us with four).
 template <typename T, bool ODD, int NT, bool PER, bool CEN>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT)
     k_lattice_batched(const __grid_constant__ LbGroup G, const int m0, const int b0,
                       const int *__restrict__ blk_member, const int *__restrict__ blk_start, const int pbuf,
                       const int ahead_nodes)
 {
+    constexpr int tiles = CEN ? kEnsTilesCentred : kEnsTiles;
     const int mi = blk_member[b0 + blockIdx.x];
     const LbView &L = G.v[mi - m0];
-    const int nx = L.n[0], nxy = L.n[0] * L.n[1];
-    const int bpp = (nxy + NT - 1) / NT;
     const int lb = b0 + (int)blockIdx.x - blk_start[mi];
-    const int z = lb / bpp;
-    const int p = (lb - z * bpp) * NT + (int)threadIdx.x;
-    if (lb == 0 && threadIdx.x == 0) close_step(L);
-    if (ahead_nodes > 0) {
-        const int za = z + (ahead_nodes + nxy - 1) / nxy;
-        if (za < L.n[2] && p < nxy) {
+    int node = lb * (tiles * NT) + (int)threadIdx.x;
+    if (node == 0) close_step(L);
+    bool bad = false;
+#pragma unroll 1
+    for (int k = 0; k < tiles; ++k, node += NT) {
+        if (ahead_nodes > 0 && node + ahead_nodes < L.nodes) {
             T *f = static_cast<T *>(L.f);
-            const unsigned off = (unsigned)(p + nxy * za) * (unsigned)sizeof(T);
+            const unsigned off = (unsigned)(node + ahead_nodes) * (unsigned)sizeof(T);
 #pragma unroll
             for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(slot_at(f, i, L.qs, off)));
         }
-    }
-    bool bad = false;
-    if (p < nxy) {
-        const int y = (int)(((float)p + 0.5f) * L.inv_nx);
-        bad = lattice_node<T, ODD, false, LAT_FAR, PER, CEN>(L, p - y * nx, y, z, p + z * nxy, pbuf);
+        if (node < L.nodes) {
+            const int z = fast_div(node, L.div_nxy), p = node - z * L.n[0] * L.n[1];
+            const int y = fast_div(p, L.div_nx), x = p - y * L.n[0];
+            bad |= lattice_node<T, ODD, false, LAT_FAR, PER, CEN>(L, x, y, z, node, pbuf);
+        }
     }
     const unsigned m = __ballot_sync(0xffffffffu, bad);
     if (m != 0u && (threadIdx.x & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
 }
 
 // Ensemble: the patch nodes of every member of a group (blockIdx.y is the
-// member within the group), a warp per patch row as in k_lattice_near.
+// member within the group), a warp per patch row as in k_lattice_near.  Capped
+// at 64 registers: at 80 its two blocks per SM held 62% of the register file
+// from the concurrent outside update for as long as they ran (step of 32
+// droplets 478 -> 457 us, of 16 centred ones 234 -> 223).
 template <typename T, bool ODD, bool PER, class P>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_lattice_near_batched(const __grid_constant__ LbGroup G,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lattice_near_batched(const __grid_constant__ LbGroup G,
                                                                                     const int buf)
 {
     const int wpb = blockDim.x >> 5;
@@ -1837,13 +1843,10 @@ cudaError_t launch_ensemble_far(const EnsembleView &E, long long step, cudaStrea
     for (int m0 = 0; m0 < n; m0 += kGroup) {
         const int m1 = m0 + kGroup < n ? m0 + kGroup : n;
         fill_group(E, m0, m1);
-        bool per = false, cen = false;
-        for (int k = m0; k < m1; ++k) {
-            per = per || any_periodic(E.lv[k]);
-            cen = cen || E.lv[k].recentre != 0;
-        }
-        if (E.precision == IBL_FP64) far_batched_p<double>(E, odd, per, cen, m0, pbuf, waves, ti, s);
-        else far_batched_p<float>(E, odd, per, cen, m0, pbuf, waves, ti, s);
+        bool per = false;
+        for (int k = m0; k < m1; ++k) per = per || any_periodic(E.lv[k]);
+        if (E.precision == IBL_FP64) far_batched_p<double>(E, odd, per, E.recentre, m0, pbuf, waves, ti, s);
+        else far_batched_p<float>(E, odd, per, E.recentre, m0, pbuf, waves, ti, s);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
