@@ -518,26 +518,30 @@ __device__ __forceinline__ void close_step(const LbView &L)
 // instructions per warp against 643 / 765 before.  Per step: 97 x 75 x 61
 // channel 16.5 -> 12.3 us, 200^3 regularised 228 -> 212 us, 128^3 droplet
 // 57.1 -> 55.0 us, 256^3 within 0.3%.
-template <typename T, bool ODD, bool REC, int MODE, bool PER, bool CEN>
+// TILES: blocks take that many tiles in turn.
+template <typename T, bool ODD, bool REC, int MODE, bool PER, bool CEN, int TILES>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 4) k_lattice(LbView L, int pbuf, int ahead)
 {
-    const int node = (int)(blockIdx.x * 128u + threadIdx.x);
+    int node = (int)(blockIdx.x * (128u * TILES) + threadIdx.x);
     if (node == 0) close_step(L);
-    // L2 prefetch of the node `ahead` nodes on, which a block of about one
-    // resident wave later updates: its loads then find the lines in L2
-    // instead of waiting on DRAM behind the stream (ahead = 0: none; the host
-    // leaves it out for a large droplet patch, see L.prefetch)
-    if (ahead > 0 && node + ahead < L.nodes) {
-        T *f = static_cast<T *>(L.f);
-        const unsigned off = (unsigned)(node + ahead) * (unsigned)sizeof(T);
-#pragma unroll
-        for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(slot_at(f, i, L.qs, off)));
-    }
     bool bad = false;
-    if (node < L.nodes) {
-        const int z = fast_div(node, L.div_nxy), p = node - z * L.n[0] * L.n[1];
-        const int y = fast_div(p, L.div_nx), x = p - y * L.n[0];
-        bad = lattice_node<T, ODD, REC, MODE, PER, CEN>(L, x, y, z, node, pbuf);
+#pragma unroll 1
+    for (int k = 0; k < TILES; ++k, node += 128) {
+        // L2 prefetch of the node `ahead` nodes on, which a block of about one
+        // resident wave later updates: its loads then find the lines in L2
+        // instead of waiting on DRAM behind the stream (ahead = 0: none, see
+        // prefetch_distance)
+        if (ahead > 0 && node + ahead < L.nodes) {
+            T *f = static_cast<T *>(L.f);
+            const unsigned off = (unsigned)(node + ahead) * (unsigned)sizeof(T);
+#pragma unroll
+            for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(slot_at(f, i, L.qs, off)));
+        }
+        if (node < L.nodes) {
+            const int z = fast_div(node, L.div_nxy), p = node - z * L.n[0] * L.n[1];
+            const int y = fast_div(p, L.div_nx), x = p - y * L.n[0];
+            bad |= lattice_node<T, ODD, REC, MODE, PER, CEN>(L, x, y, z, node, pbuf);
+        }
     }
     // sticky instability flag, one atomic per warp at most
     const unsigned m = __ballot_sync(0xffffffffu, bad);
@@ -1458,29 +1462,55 @@ static bool any_periodic(const LbView &L)
     return L.bc[0] == IBL_BC_PERIODIC || L.bc[1] == IBL_BC_PERIODIC || L.bc[2] == IBL_BC_PERIODIC;
 }
 
+// Prefetch distance in nodes: one wave of resident blocks; none where the host
+// left it out beside a large droplet patch (L.prefetch), nor for populations
+// that stay in L2 between steps (up to 96 MB of its 129), where the 19
+// prefetches only cost issue slots (97 x 75 x 61 channel 12.3 -> 11.7 us a
+// step; 128^3, 159 MB, keeps them: 51.8 us with, 53.7 without).
+template <typename T>
+static int prefetch_distance(const LbView &L)
+{
+    if (!L.prefetch || 19 * L.qs * (long long)sizeof(T) <= (96ll << 20)) return 0;
+    return sm_count() * (sizeof(T) == 4 ? 8 : 4) * 128;
+}
+
+// Tiles per block of the update outside a droplet patch.  Beside a droplet in
+// a small FP32 box the chain of droplet kernels sets the step, and it waits
+// for SM slots: a quarter of the blocks leaves every SM slots free (us per
+// step with one and four tiles: 48^3 12.8 and 11.4, 56^3 14.9 and 11.9, 64^3
+// 17.0 and 15.0, 72^3 17.9 and 15.9, 80^3 19.0 and 18.1, 88^3 20.0 and 21.0,
+// 128^3 55.0 and 57.8).  Without a droplet one tile is faster at every size,
+// and FP64 needs every SM's FP64 pipe.
+constexpr int kFarTiles = 4, kFarTilesNodes = 80 * 80 * 80;
+
 // Variants: a recording launch takes the general (periodic) form, and CEN
 // (re-centring) exists only where a droplet does.
 template <typename T, bool ODD>
 static void lattice_launch_t(const LbView &L, bool rec, int mode, int pbuf, cudaStream_t s)
 {
-    const unsigned g = blocks_for(L.nodes, 128);
-    // prefetch distance: the nodes one wave of resident blocks covers
-    const int ahead = L.prefetch ? sm_count() * (sizeof(T) == 4 ? 8 : 4) * 128 : 0;
+    const int ahead = prefetch_distance<T>(L);
     const bool per = any_periodic(L), cen = L.recentre != 0;
-#define IBL_LAUNCH(R, M, P, C) k_lattice<T, ODD, R, M, P, C><<<g, 128, 0, s>>>(L, pbuf, ahead)
+    const bool tiled = sizeof(T) == 4 && L.nodes <= kFarTilesNodes;
+#define IBL_LAUNCH(R, M, P, C, K) \
+    k_lattice<T, ODD, R, M, P, C, K><<<blocks_for(L.nodes, 128 * K), 128, 0, s>>>(L, pbuf, ahead)
+#define IBL_LAUNCH_FAR(P, C)                                                    \
+    do {                                                                        \
+        if (rec) IBL_LAUNCH(true, LAT_FAR, true, C, 1);                         \
+        else if (sizeof(T) == 4 && tiled) IBL_LAUNCH(false, LAT_FAR, P, C, (sizeof(T) == 4 ? kFarTiles : 1)); \
+        else IBL_LAUNCH(false, LAT_FAR, P, C, 1);                               \
+    } while (0)
     if (mode != LAT_FAR) {
-        if (rec) IBL_LAUNCH(true, LAT_FULL, true, false);
-        else if (per) IBL_LAUNCH(false, LAT_FULL, true, false);
-        else IBL_LAUNCH(false, LAT_FULL, false, false);
+        if (rec) IBL_LAUNCH(true, LAT_FULL, true, false, 1);
+        else if (per) IBL_LAUNCH(false, LAT_FULL, true, false, 1);
+        else IBL_LAUNCH(false, LAT_FULL, false, false, 1);
     } else if (cen) {
-        if (rec) IBL_LAUNCH(true, LAT_FAR, true, true);
-        else if (per) IBL_LAUNCH(false, LAT_FAR, true, true);
-        else IBL_LAUNCH(false, LAT_FAR, false, true);
+        if (per) IBL_LAUNCH_FAR(true, true);
+        else IBL_LAUNCH_FAR(false, true);
     } else {
-        if (rec) IBL_LAUNCH(true, LAT_FAR, true, false);
-        else if (per) IBL_LAUNCH(false, LAT_FAR, true, false);
-        else IBL_LAUNCH(false, LAT_FAR, false, false);
+        if (per) IBL_LAUNCH_FAR(true, false);
+        else IBL_LAUNCH_FAR(false, false);
     }
+#undef IBL_LAUNCH_FAR
 #undef IBL_LAUNCH
 }
 
