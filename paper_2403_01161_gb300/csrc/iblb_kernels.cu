@@ -163,12 +163,13 @@ __device__ __forceinline__ void bc_apply(T (&f)[19], const T (&uw)[3], int rule)
     }
 }
 
-template <typename T>
+// MIRRORED: no case on the x = nx - 1 wall.
+template <typename T, bool MIRRORED>
 __device__ __forceinline__ void bc_dispatch(T (&f)[19], const T (&uw)[3], int rule, int code)
 {
-#define IBL_BC_CASE(a, b, c)                              \
-    case (a + 1) + 3 * (b + 1) + 9 * (c + 1):             \
-        bc_apply<T, a, b, c>(f, uw, rule);                \
+#define IBL_BC_CASE(a, b, c)                                              \
+    case (a + 1) + 3 * (b + 1) + 9 * (c + 1):                             \
+        if constexpr (!(MIRRORED && a > 0)) bc_apply<T, a, b, c>(f, uw, rule); \
         break;
     switch (code) {
         IBL_BC_CASE(-1, 0, 0) IBL_BC_CASE(1, 0, 0) IBL_BC_CASE(0, -1, 0) IBL_BC_CASE(0, 1, 0)
@@ -213,6 +214,167 @@ __device__ __forceinline__ T odd_weight()
 {
     if constexpr (sizeof(T) == 4) return __int_as_float(c2(i) == 1 ? 0x3E2AAAAA : 0x3DAAAAAB);
     else return T(3.0 * wgt(i));
+}
+
+// Moments with half-force momentum, BGK and Guo source (FORCE) on the 19
+// populations of a node, in place; returns whether it is unstable.  FP32: each
+// population is relaxed from its own value, and the momentum terms keep the
+// weights of odd_weight.
+template <bool FORCE, typename T>
+__device__ __forceinline__ bool collide(T (&g)[19], const T Fx, const T Fy, const T Fz, const T om, T &drho, T &ux, T &uy,
+                                        T &uz)
+{
+    drho = T(0);
+    T jx = T(0), jy = T(0), jz = T(0);
+    sfor<19>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        drho += g[i];
+        if constexpr (cxf(i) != 0) jx += T(cxf(i)) * g[i];
+        if constexpr (cyf(i) != 0) jy += T(cyf(i)) * g[i];
+        if constexpr (czf(i) != 0) jz += T(czf(i)) * g[i];
+    });
+    const T rho = T(1) + drho;
+    const T ir = T(1) / rho;
+    // rho u = j + F/2 (Eq. (density_velocity_LB)); the odd (momentum)
+    // parts of the equilibrium are formed from it directly
+    T mx = jx, my = jy, mz = jz;
+    if constexpr (FORCE) {
+        mx += T(0.5) * Fx;
+        my += T(0.5) * Fy;
+        mz += T(0.5) * Fz;
+    }
+    ux = mx * ir;
+    uy = my * ir;
+    uz = mz * ir;
+    const T uu = ux * ux + uy * uy + uz * uz;
+    const bool bad = !(uu <= T(0.09)) || !(drho == drho);
+    [[maybe_unused]] T fpre, uF;
+    if constexpr (FORCE) {
+        fpre = T(1) - T(0.5) * om;
+        uF = ux * Fx + uy * Fy + uz * Fz;
+    }
+    const T dmr = drho - rho * (T(1.5) * uu);  // drho - (3/2) rho u.u
+    {
+        constexpr double w0 = wgt(0);
+        const T geq = T(w0) * dmr;
+        g[0] = g[0] + om * (geq - g[0]);
+        if constexpr (FORCE) g[0] += fpre * T(w0) * (T(-3) * uF);
+    }
+    sfor<9>([&](auto I) {
+        constexpr int i = decltype(I)::value + 1;
+        constexpr int j = opp(i);
+        T cp = T(0);  // c_i . rho u
+        if constexpr (cxf(i) != 0) cp += T(cxf(i)) * mx;
+        if constexpr (cyf(i) != 0) cp += T(cyf(i)) * my;
+        if constexpr (czf(i) != 0) cp += T(czf(i)) * mz;
+        const T cu = cp * ir;
+        constexpr double w = wgt(i);
+        const T w3 = odd_weight<T, i>();
+        const T even_eq = T(w) * (T(4.5) * cp * cu + dmr);
+        const T odd_eq = w3 * cp;
+        g[i] = g[i] + om * (even_eq + odd_eq - g[i]);
+        g[j] = g[j] + om * (even_eq - odd_eq - g[j]);
+        if constexpr (FORCE) {
+            T cF = T(0);  // c_i . F
+            if constexpr (cxf(i) != 0) cF += T(cxf(i)) * Fx;
+            if constexpr (cyf(i) != 0) cF += T(cyf(i)) * Fy;
+            if constexpr (czf(i) != 0) cF += T(czf(i)) * Fz;
+            const T even_src = fpre * T(w) * (T(9) * cu * cF - T(3) * uF);
+            const T odd_src = fpre * w3 * cF;
+            g[i] += even_src + odd_src;
+            g[j] += even_src - odd_src;
+        }
+    });
+    return bad;
+}
+
+// FP64: the same on sums and differences of opposite populations, s = g_i +
+// g_j and d = g_i - g_j: the moments need each once, and a pair relaxes as
+//   g_i, g_j = [(1 - w)/2 s + w even_eq] +- [(1 - w)/2 d + w odd_eq]
+// (w = omega), 143 FP64 instructions a node without force against 185: the
+// FP64 pipe, one warp instruction per 16 cycles and SM, sets the FP64 step.
+// (FP32 keeps `collide`: there this grouping rounds the momentum worse.)  u is
+// formed only where it is stored (VEL).
+template <bool FORCE, bool VEL, typename T>
+__device__ __forceinline__ bool collide_pairs(T (&g)[19], const T Fx, const T Fy, const T Fz, const T om, T &drho, T &ux,
+                                              T &uy, T &uz)
+{
+    drho = g[0];
+    T mx = T(0), my = T(0), mz = T(0);  // rho u
+    if constexpr (FORCE) {
+        mx = T(0.5) * Fx;
+        my = T(0.5) * Fy;
+        mz = T(0.5) * Fz;
+    }
+    sfor<9>([&](auto I) {
+        constexpr int i = decltype(I)::value + 1, j = opp(i);
+        const T s = g[i] + g[j], d = g[i] - g[j];
+        g[i] = s;
+        g[j] = d;
+        drho += s;
+        if constexpr (cxf(i) != 0) mx += T(cxf(i)) * d;
+        if constexpr (cyf(i) != 0) my += T(cyf(i)) * d;
+        if constexpr (czf(i) != 0) mz += T(czf(i)) * d;
+    });
+    const T ir = T(1) / (T(1) + drho);
+    const T ke = (mx * mx + my * my + mz * mz) * ir;  // rho u.u
+    const bool bad = !(ke * ir <= T(0.09));           // NaN density included
+    const T dmr = drho - T(1.5) * ke, q = T(4.5) * ir;
+    const T keep = T(0.5) - T(0.5) * om;
+    [[maybe_unused]] T fpre, uF;
+    if constexpr (VEL) {
+        ux = mx * ir;
+        uy = my * ir;
+        uz = mz * ir;
+    }
+    if constexpr (FORCE) {
+        fpre = T(1) - T(0.5) * om;
+        uF = ux * Fx + uy * Fy + uz * Fz;
+    }
+    g[0] = (keep + keep) * g[0] + (om * T(wgt(0))) * dmr;
+    if constexpr (FORCE) g[0] -= (fpre * T(3.0 * wgt(0))) * uF;
+    const T e1 = om * T(wgt(1)), e2 = om * T(wgt(4)), o1 = om * T(3.0 * wgt(1)), o2 = om * T(3.0 * wgt(4));
+    sfor<9>([&](auto I) {
+        constexpr int i = decltype(I)::value + 1, j = opp(i);
+        constexpr bool axis = c2(i) == 1;
+        T cp = T(0);  // c_i . rho u
+        if constexpr (cxf(i) != 0) cp += T(cxf(i)) * mx;
+        if constexpr (cyf(i) != 0) cp += T(cyf(i)) * my;
+        if constexpr (czf(i) != 0) cp += T(czf(i)) * mz;
+        T S = keep * g[i] + (axis ? e1 : e2) * (q * (cp * cp) + dmr);
+        T D = keep * g[j] + (axis ? o1 : o2) * cp;
+        if constexpr (FORCE) {
+            T cF = T(0);  // c_i . F
+            if constexpr (cxf(i) != 0) cF += T(cxf(i)) * Fx;
+            if constexpr (cyf(i) != 0) cF += T(cyf(i)) * Fy;
+            if constexpr (czf(i) != 0) cF += T(czf(i)) * Fz;
+            S += fpre * T(wgt(i)) * (T(9) * (cp * ir) * cF - T(3) * uF);
+            D += fpre * T(3.0 * wgt(i)) * cF;
+        }
+        g[i] = S + D;
+        g[j] = S - D;
+    });
+    return bad;
+}
+
+// Population of the velocity c_i with its x component reversed.
+__host__ __device__ constexpr int mirrored(int i)
+{
+    for (int j = 0; j < 19; ++j)
+        if (cxf(j) == -cxf(i) && cyf(j) == cyf(i) && czf(j) == czf(i)) return j;
+    return i;
+}
+template <typename T>
+__device__ __forceinline__ void mirror_x(T (&g)[19], const bool on)
+{
+    sfor<19>([&](auto I) {
+        constexpr int i = decltype(I)::value, j = mirrored(i);
+        if constexpr (cxf(i) > 0) {
+            const T a = g[i], b = g[j];
+            g[i] = on ? b : a;
+            g[j] = on ? a : b;
+        }
+    });
 }
 
 // Byte offsets to a node's neighbours along each axis (odd step).  Periodic
@@ -315,7 +477,19 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
             }
             const T uw[3] = {A[0] * lx + A[1] * ly + A[2] * lz, A[3] * lx + A[4] * ly + A[5] * lz,
                              A[6] * lx + A[7] * ly + A[8] * lz};
-            bc_dispatch<T>(g, uw, L.rule, (sx + 1) + 3 * (sy + 1) + 9 * (sz + 1));
+            if constexpr (sizeof(T) == 4) {
+                bc_dispatch<T, false>(g, uw, L.rule, (sx + 1) + 3 * (sy + 1) + 9 * (sz + 1));
+            } else {
+                // both x walls through one rebuild, the far one mirrored: a
+                // warp that holds both (rows of 32 nodes and fewer, or rows
+                // that are no multiple of 32) issues its FP64 instructions
+                // once; the exchange is selects
+                const bool mir = sx > 0;
+                const T vw[3] = {mir ? -uw[0] : uw[0], uw[1], uw[2]};
+                mirror_x(g, mir);
+                bc_dispatch<T, true>(g, vw, L.rule, (mir ? 0 : sx + 1) + 3 * (sy + 1) + 9 * (sz + 1));
+                mirror_x(g, mir);
+            }
         }
 
         // droplet patch: read the spread force (and clear it), store u below;
@@ -327,27 +501,6 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
             K.st3(force + 4 * node, T(0), T(0), T(0));
         }
 
-        T drho = T(0), jx = T(0), jy = T(0), jz = T(0);
-        sfor<19>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            drho += g[i];
-            if constexpr (cxf(i) != 0) jx += T(cxf(i)) * g[i];
-            if constexpr (cyf(i) != 0) jy += T(cyf(i)) * g[i];
-            if constexpr (czf(i) != 0) jz += T(czf(i)) * g[i];
-        });
-        const T rho = T(1) + drho;
-        const T ir = T(1) / rho;
-        // rho u = j + F/2 (Eq. (density_velocity_LB)); the odd (momentum)
-        // parts of the equilibrium are formed from it directly
-        T mx = jx, my = jy, mz = jz;
-        if constexpr (FORCE) {
-            mx += T(0.5) * Fx;
-            my += T(0.5) * Fy;
-            mz += T(0.5) * Fz;
-        }
-        const T ux = mx * ir, uy = my * ir, uz = mz * ir;
-        const T uu = ux * ux + uy * uy + uz * uz;
-        bad = !(uu <= T(0.09)) || !(drho == drho);
         T om = sizeof(T) == 4 ? T(L.omega_f) : T(L.omega);
         if constexpr (MODE == LAT_NEAR) {
             // viscosity ratio: relaxation of the inside nodes (flags read and cleared)
@@ -357,43 +510,9 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
                 *flag = 0;
             }
         }
-        [[maybe_unused]] T fpre, uF;
-        if constexpr (FORCE) {
-            fpre = T(1) - T(0.5) * om;
-            uF = ux * Fx + uy * Fy + uz * Fz;
-        }
-        const T dmr = drho - rho * (T(1.5) * uu);  // drho - (3/2) rho u.u
-        {
-            constexpr double w0 = wgt(0);
-            const T geq = T(w0) * dmr;
-            g[0] = g[0] + om * (geq - g[0]);
-            if constexpr (FORCE) g[0] += fpre * T(w0) * (T(-3) * uF);
-        }
-        sfor<9>([&](auto I) {
-            constexpr int i = decltype(I)::value + 1;
-            constexpr int j = opp(i);
-            T cp = T(0);  // c_i . rho u
-            if constexpr (cxf(i) != 0) cp += T(cxf(i)) * mx;
-            if constexpr (cyf(i) != 0) cp += T(cyf(i)) * my;
-            if constexpr (czf(i) != 0) cp += T(czf(i)) * mz;
-            const T cu = cp * ir;
-            constexpr double w = wgt(i);
-            const T w3 = odd_weight<T, i>();
-            const T even_eq = T(w) * (T(4.5) * cp * cu + dmr);
-            const T odd_eq = w3 * cp;
-            g[i] = g[i] + om * (even_eq + odd_eq - g[i]);
-            g[j] = g[j] + om * (even_eq - odd_eq - g[j]);
-            if constexpr (FORCE) {
-                T cF = T(0);  // c_i . F
-                if constexpr (cxf(i) != 0) cF += T(cxf(i)) * Fx;
-                if constexpr (cyf(i) != 0) cF += T(cyf(i)) * Fy;
-                if constexpr (czf(i) != 0) cF += T(czf(i)) * Fz;
-                const T even_src = fpre * T(w) * (T(9) * cu * cF - T(3) * uF);
-                const T odd_src = fpre * w3 * cF;
-                g[i] += even_src + odd_src;
-                g[j] += even_src - odd_src;
-            }
-        });
+        T drho, ux, uy, uz;
+        if constexpr (sizeof(T) == 4) bad = collide<FORCE>(g, Fx, Fy, Fz, om, drho, ux, uy, uz);
+        else bad = collide_pairs<FORCE, FORCE || REC>(g, Fx, Fy, Fz, om, drho, ux, uy, uz);
 
         if constexpr (!ODD) {
             sfor<19>([&](auto I) {
