@@ -614,6 +614,14 @@ __device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const
     }
 }
 
+// Sets the sticky instability flag.  Once it is set, further warps only look
+// (a line their SM has cached): a box that has gone unstable has every warp
+// here at every step, all on one address.
+__device__ __forceinline__ void flag_unstable(const LbView &L)
+{
+    if ((L.ctl->err & IBL_ERRBIT_UNSTABLE) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
+}
+
 // Closes step t: the step counter becomes t + 1 and the frame of step t + 1
 // goes to its parity's slot.  The lattice kernel of step t and the patch
 // update of step t read the other slot, and the kernels of step t - 1, the
@@ -664,7 +672,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 4) k_lattice(LbView 
     }
     // sticky instability flag, one atomic per warp at most
     const unsigned m = __ballot_sync(0xffffffffu, bad);
-    if (m != 0u && (threadIdx.x & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
+    if (m != 0u && (threadIdx.x & 31) == 0) flag_unstable(L);
 }
 
 // Outside update (FAR) or whole-box update (FULL) through a shared-memory
@@ -823,7 +831,7 @@ __global__ void __launch_bounds__(NT, (B > 768 / NT ? B : 768 / NT)) k_lattice_s
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, bad);
-        if (m != 0u && (tid & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
+        if (m != 0u && (tid & 31) == 0) flag_unstable(L);
         __syncthreads();  // every thread is done with stage s
         if (tid < 32) {
             const int t = tile + S * (int)gridDim.x;
@@ -859,7 +867,7 @@ __device__ __forceinline__ void patch_rows(const LbView &L, const int buf, const
                 bad = lattice_node<T, ODD, REC, LAT_NEAR, PER, true, P>(L, x, y, z, x + L.n[0] * (y + L.n[1] * z), buf);
             }
             const unsigned m = __ballot_sync(0xffffffffu, bad);
-            if (m != 0u && lane == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
+            if (m != 0u && lane == 0) flag_unstable(L);
         }
     }
 }
@@ -916,7 +924,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT)
         }
     }
     const unsigned m = __ballot_sync(0xffffffffu, bad);
-    if (m != 0u && (threadIdx.x & 31) == 0) atomicOr(&L.ctl->err, IBL_ERRBIT_UNSTABLE);
+    if (m != 0u && (threadIdx.x & 31) == 0) flag_unstable(L);
 }
 
 // Ensemble: the patch nodes of every member of a group (blockIdx.y is the
