@@ -2350,26 +2350,24 @@ int ibl_adjoint(ibl_lb *lb, long long n_steps, int K, void *workspace, size_t by
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s_rec, ev[12], 0);
         if (e != cudaSuccess) st = cuda_fail(e, "adjoint seed");
     }
-    // Capture every graph the sweep below will replay while the GPU runs the
-    // forward pass just enqueued (capture and instantiation are host work).
-    {
-        int c = cur;
-        for (long long sg = last; sg >= 0 && st == IBL_OK; --sg) {
-            const int len = (int)std::min<long long>(K, n_steps - sg * K);
-            if (len == K) st = reverse_graph(c, (int)(sg & 1));
-            if (st == IBL_OK && sg >= 1) st = record_graph((sg - 1) * K, false, (int)((sg - 1) & 1), nullptr);
-            c ^= (len & 1);
-        }
-    }
     // Reverse sweep, last segment first.  While segment sg is swept back on
     // the main stream, segment sg - 1 is restored from its checkpoint and
     // recorded on its own stream into the other slot set; it waits for the
     // sweep of sg + 1, which used that set.  Both chains are latency-bound,
     // so they share the GPU well.
+    // The graphs a segment needs (its sweep's and the next recording's) are
+    // captured just before it is enqueued: the first ones while the GPU runs
+    // the forward pass just enqueued, the others while it sweeps the segments
+    // before (capture and instantiation are host work, about 2 ms per 100
+    // steps; all of them ahead of the sweep left the GPU idle for 5 of the 33
+    // ms of a 600-step call).
     for (long long sg = last; sg >= 0 && st == IBL_OK; --sg) {
         const long long t0 = sg * K;
         const int len = (int)std::min<long long>(K, n_steps - t0);
         const int set = (int)(sg & 1);
+        if (len == K) st = reverse_graph(cur, set);
+        if (st == IBL_OK && sg >= 1) st = record_graph(t0 - K, false, (int)((sg - 1) & 1), nullptr);
+        if (st != IBL_OK) break;
         if (sg < last) {
             e = cudaStreamWaitEvent(s, ev[8 + set], 0);
             if (e != cudaSuccess) {
