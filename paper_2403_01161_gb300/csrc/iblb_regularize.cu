@@ -255,8 +255,8 @@ __device__ __forceinline__ void regularize_body(const LbView &L, const MeshView 
 
     // valence weights, this CTA's nodes and neighbour addresses
     if (tid < kRegValences) {
-        wa[tid] = tid > 0 ? oma / tid : 0.0;
-        wg[tid] = tid > 0 ? sg * omg / tid : 0.0;
+        wa[tid] = oma / tid;
+        wg[tid] = sg * omg / tid;
     }
     if (tid < 2) cta_max[tid] = 0ull;
     if (tid < 6) cta_box[tid] = 0ull;
