@@ -65,8 +65,8 @@ def _mesh(kind):
     return _tube(rings, around)
 
 
-# tube1x70: poles above the weight table; tube2x3000: one pole's list above the address table of its CTA;
-# tube127x129: 16385 - 1 + 1 nodes less one ring, close to the largest mesh; tube2x8191: exactly 16384 nodes
+# tube1x70: poles above the weight table; tube2x3000: a pole's list above the address table of its CTA;
+# tube126x129: 16256 nodes, close to the largest mesh; tube2x8191: exactly the largest, 16384 nodes
 @pytest.mark.parametrize("kind", ["level0", "level1", "level3", "tube1x70", "tube2x3000", "tube126x129", "tube2x8191"])
 @pytest.mark.parametrize("sign", [1, 0])
 def test_noalloc_against_numpy(kind, sign):
