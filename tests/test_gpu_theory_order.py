@@ -57,3 +57,22 @@ def test_axes_closer_than_fp32_resolves(delta, before):
     E = A[:, -1]
     beta = np.einsum("ti,tij,tj->t", longest, E, longest) / np.linalg.norm(E, axis=(1, 2))
     assert np.abs(out[:, 7] - beta).max() <= 100 * EPS * R ** 2 / abs(delta)
+
+
+@pytest.mark.parametrize("n_frames,first", [(20, 20), (64, 40), (100, 50), (100, 100)])
+def test_rest_under_a_step_beyond_the_stability_limit(n_frames, first):
+    """A droplet at rest stays the sphere however large the multiplier of a step is."""
+    from paper_2403_01161_gb300.theory import linear_theory
+
+    A = np.zeros((2, n_frames, 3, 3))
+    A[1, first:, 0, 1] = A[1, first:, 1, 0] = 1e-4
+    a, hold = O.lt_coefficients(CHI)[0] / TAU, 1e6 * TAU
+    z = -a * hold
+    m = 1 + z * (1 + z * (0.5 + z * (1 / 6 + z / 24)))
+    assert 1e20 < m < 1e30
+    out = linear_theory(A, TAU, R, hold, CHI, substeps=1).cpu().numpy()
+    rest = np.concatenate([out[0], out[1, :first]])
+    assert (rest[:, :3] == R * R).all() and (rest[:, 3:6] == 0).all() and (rest[:, 8] == 0).all()
+    if first < n_frames:  # the first strained frame: (1 - m) of the way to the fixed point
+        want = 2 * R * R * O.lt_coefficients(CHI)[1] * 1e-4 / a * (1 - m)
+        assert abs(out[1, first, 3] / want - 1) <= 20 * EPS
