@@ -76,3 +76,25 @@ def test_rest_under_a_step_beyond_the_stability_limit(n_frames, first):
     if first < n_frames:  # the first strained frame: (1 - m) of the way to the fixed point
         want = 2 * R * R * O.lt_coefficients(CHI)[1] * 1e-4 / a * (1 - m)
         assert abs(out[1, first, 3] / want - 1) <= 20 * EPS
+
+
+@pytest.mark.parametrize("exponent", [-300, -200, 200, 300])
+def test_observables_do_not_depend_on_the_size_of_the_droplet(exponent):
+    from paper_2403_01161_gb300.theory import linear_theory
+
+    rng = np.random.default_rng(1)
+    A = rng.standard_normal((3, 40, 3, 3)) * 1e-4
+    A -= np.trace(A, axis1=2, axis2=3)[..., None, None] / 3 * np.eye(3)
+    want = linear_theory(A, TAU, 1.0, HOLD, CHI, substeps=8).cpu().numpy()
+    out = linear_theory(A, TAU, 2.0 ** exponent, HOLD, CHI, substeps=8).cpu().numpy()
+    S = want[..., :6]
+    assert np.abs(out[..., :6] * 2.0 ** -exponent * 2.0 ** -exponent - S).max() <= 8 * EPS * S.max()
+    # the eigen-solves of the two sizes may differ: eps over the gap to the next axis
+    full = np.empty(S.shape[:-1] + (3, 3))
+    for c, (i, j) in enumerate(((0, 0), (1, 1), (2, 2), (0, 1), (0, 2), (1, 2))):
+        full[..., i, j] = full[..., j, i] = S[..., c]
+    lam = np.linalg.eigvalsh(full)
+    assert np.abs(out[..., 6] - want[..., 6]).max() <= 40 * EPS * lam.max()
+    assert np.abs(out[..., 8] - want[..., 8]).max() <= 40 * EPS * lam.max() / lam.min()
+    gap = (lam[..., 2] - lam[..., 1]) / lam[..., 2]
+    assert (np.abs(out[..., 7] - want[..., 7]) <= 80 * EPS / gap).all()
