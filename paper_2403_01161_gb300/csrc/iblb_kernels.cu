@@ -377,20 +377,34 @@ __device__ __forceinline__ void mirror_x(T (&g)[19], const bool on)
     });
 }
 
-// Byte offsets to a node's neighbours along each axis (odd step).  Periodic
-// axes wrap.  On a Zou-He axis a missing neighbour points back at the node
-// itself: a population whose source lies outside the box is an unknown that
-// the boundary rebuild overwrites before anything reads it, so its load only
-// needs an address inside the array, while a store to a missing destination
-// is left out (the flags).
+// Offsets to a node's neighbours along each axis (odd step), in units of 1/S
+// node.  Periodic axes wrap.  On a Zou-He axis a missing neighbour points back
+// at the node itself: a population whose source lies outside the box is an
+// unknown that the boundary rebuild overwrites before anything reads it, so
+// its load only needs an address inside the array, while a store to a missing
+// destination is left out: by the flags, or where an axis may be periodic by
+// the bits of `miss` (six flags beside six run-time offsets made the periodic
+// patch update of an ensemble spill 88 bytes, the bits 4).
 struct Hops {
     int xm, xp, ym, yp, zm, zp;
     bool no_xm, no_xp, no_ym, no_yp, no_zm, no_zp;
+    int miss;  // 1 x-1, 2 x+1, 4 y-1, 8 y+1, 16 z-1, 32 z+1
 };
-template <typename T, bool PER>
+// Whether an odd update forms its addresses from element indices and its hops
+// twice, before the loads and again for the stores, instead of byte offsets on
+// common bases held across the collision.  Outside the patch of a box with a
+// periodic axis, where the hops are selects at run time, that is fewer
+// instructions and registers (FP32, us per step, byte offsets and indices:
+// periodic 128^3 droplet 53.1 and 50.7, 160^3 100.4 and 97.3, 256^3 412.6 and
+// 403.5, 64^3 12.37 and 12.45; channel without a droplet 64^3 6.06 and 5.59,
+// 256^3 372.1 and 372.7; 32 periodic droplets 358.4 and 348.3).  FP64, set by
+// its pipe, does not gain (64^3 droplet 94.0 and 94.7).
+template <typename T, int MODE, bool PER>
+constexpr bool kIndexed = sizeof(T) == 4 && PER && MODE != LAT_NEAR;
+template <int S, bool PER>
 __device__ __forceinline__ Hops make_hops(const LbView &L, const int x, const int y, const int z)
 {
-    const int nx = L.n[0], ny = L.n[1], nz = L.n[2], S = (int)sizeof(T), Sx = S * nx, Sxy = Sx * ny;
+    const int nx = L.n[0], ny = L.n[1], nz = L.n[2], Sx = S * nx, Sxy = Sx * ny;
     const bool px = PER && L.bc[0] == IBL_BC_PERIODIC, py = PER && L.bc[1] == IBL_BC_PERIODIC,
                pz = PER && L.bc[2] == IBL_BC_PERIODIC;
     Hops h;
@@ -414,6 +428,8 @@ __device__ __forceinline__ Hops make_hops(const LbView &L, const int x, const in
         h.no_zm = h.no_zm && !pz;
         h.no_zp = h.no_zp && !pz;
     }
+    h.miss = (h.no_xm ? 1 : 0) | (h.no_xp ? 2 : 0) | (h.no_ym ? 4 : 0) | (h.no_yp ? 8 : 0) | (h.no_zm ? 16 : 0) |
+             (h.no_zp ? 32 : 0);
     return h;
 }
 // Offset of the neighbour along (CX, CY, CZ), and whether it exists.
@@ -426,9 +442,14 @@ __device__ __forceinline__ unsigned hop(const Hops &h)
     if constexpr (CZ != 0) o += (unsigned)(CZ > 0 ? h.zp : h.zm);
     return o;
 }
-template <int CX, int CY, int CZ>
+template <bool PER, int CX, int CY, int CZ>
 __device__ __forceinline__ bool hop_exists(const Hops &h)
 {
+    if constexpr (PER) {
+        constexpr int need = (CX > 0 ? 2 : (CX < 0 ? 1 : 0)) | (CY > 0 ? 8 : (CY < 0 ? 4 : 0)) |
+                             (CZ > 0 ? 32 : (CZ < 0 ? 16 : 0));
+        return (h.miss & need) == 0;
+    }
     bool no = false;
     if constexpr (CX != 0) no = no || (CX > 0 ? h.no_xp : h.no_xm);
     if constexpr (CY != 0) no = no || (CY > 0 ? h.no_yp : h.no_ym);
@@ -524,22 +545,26 @@ __device__ __forceinline__ bool lattice_finish(const LbView &L, T (&g)[19], cons
             // destination x + c_i, slot i.  The node's own offset passes
             // through an opaque move, so the neighbour offsets are summed
             // again here instead of being held in registers across the
-            // collision; the patch-node update, which holds more, forms them
-            // anew from the coordinates (either way the kernel spilled).
+            // collision; the patch-node update, which holds more, and the
+            // indexed one form them anew from the coordinates (either way the
+            // kernel spilled).
+            constexpr bool IDX = kIndexed<T, MODE, PER>;
             unsigned here = noff;
-            asm volatile("mov.b32 %0, %0;" : "+r"(here));
             Hops h = h_;
-            if constexpr (MODE == LAT_NEAR) {
+            if constexpr (MODE == LAT_NEAR || IDX) {
                 int xs = x, ys = y, zs = z;
                 asm volatile("mov.b32 %0, %0;" : "+r"(xs));
                 asm volatile("mov.b32 %0, %0;" : "+r"(ys));
                 asm volatile("mov.b32 %0, %0;" : "+r"(zs));
-                h = make_hops<T, PER>(L, xs, ys, zs);
+                h = make_hops<IDX ? 1 : (int)sizeof(T), PER>(L, xs, ys, zs);
+                if constexpr (IDX) here = (unsigned)(xs + nx * (ys + ny * zs));
             }
+            if constexpr (!IDX) asm volatile("mov.b32 %0, %0;" : "+r"(here));
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                if (hop_exists<cxf(i), cyf(i), czf(i)>(h)) {
-                    T *a = slot_at(f, i, qs, here + hop<cxf(i), cyf(i), czf(i)>(h));
+                if (hop_exists<PER, cxf(i), cyf(i), czf(i)>(h)) {
+                    const unsigned o = here + hop<cxf(i), cyf(i), czf(i)>(h);
+                    T *a = IDX ? f + (i * (int)qs + (int)o) : slot_at(f, i, qs, o);
                     if constexpr (MODE == LAT_NEAR) K.st(a, g[i]);
                     else *a = g[i];
                 }
@@ -575,7 +600,6 @@ __device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const
         if (node_in_patch<PER>(L, L.ctl, pbuf, x, y, z)) return false;
     }
     {
-        const int nxy = nx * ny;
         T *__restrict__ f = static_cast<T *>(L.f);
         // the patch nodes keep their lines in L2 between steps (see L2Keep)
         struct NoKeep {};
@@ -588,7 +612,8 @@ __device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const
         const int sz = pz ? 0 : (z == 0 ? -1 : (z == nz - 1 ? 1 : 0));
         // the patch-node update guards its loads too, which measured faster there
         [[maybe_unused]] Hops h{};
-        if constexpr (ODD) h = make_hops<T, PER>(L, x, y, z);
+        constexpr bool IDX = kIndexed<T, MODE, PER>;
+        if constexpr (ODD) h = make_hops<IDX ? 1 : (int)sizeof(T), PER>(L, x, y, z);
         [[maybe_unused]] const unsigned noff = (unsigned)node * (unsigned)sizeof(T);
 
         T g[19];
@@ -603,9 +628,10 @@ __device__ __forceinline__ bool lattice_node(const LbView &L, const int x, const
             // source x - c_i, slot opp(i)
             sfor<19>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                const T *a = slot_at(f, opp(i), qs, noff + hop<-cxf(i), -cyf(i), -czf(i)>(h));
+                const unsigned o = hop<-cxf(i), -cyf(i), -czf(i)>(h);
+                const T *a = IDX ? f + (opp(i) * (int)qs + node + (int)o) : slot_at(f, opp(i), qs, noff + o);
                 if constexpr (MODE == LAT_NEAR)
-                    g[i] = hop_exists<-cxf(i), -cyf(i), -czf(i)>(h) ? K.ld(a) : T(0);
+                    g[i] = hop_exists<PER, -cxf(i), -cyf(i), -czf(i)>(h) ? K.ld(a) : T(0);
                 else g[i] = *a;
             });
         }
@@ -826,7 +852,7 @@ __global__ void __launch_bounds__(NT, (B > 768 / NT ? B : 768 / NT)) k_lattice_s
                     else g[i] = src[i * RUN];
                 });
                 Hops h{};
-                if constexpr (ODD) h = make_hops<float, false>(L, x, y, z);
+                if constexpr (ODD) h = make_hops<(int)sizeof(float), false>(L, x, y, z);
                 bad = lattice_finish<float, ODD, false, MODE, false, true>(L, g, x, y, z, n, pbuf, sx, sy, sz, h);
             }
         }
