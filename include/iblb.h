@@ -348,13 +348,28 @@ int ibl_regularize_now(ibl_mesh *m, int *iters);
  * int32, one-ring neighbours as returned by ibl_copy_neighbours), and
  * result (2 int32: iterations, 1 if converged else 0).  Asynchronous on
  * `stream` (a cudaStream_t, NULL = legacy default stream).
- * Scratch: the shared memory of one thread-block cluster; n_nodes above
- * 16384 is rejected with IBL_EINVAL.  No device memory is held between calls,
- * and calls on different buffers may overlap.  Make the first call on each
- * device outside a stream capture (it asks the device for its cluster
- * sizes).  Calls no allocating routine. */
+ * Scratch: the shared memory of one thread-block cluster of 16 or 8 blocks;
+ * n_nodes above 16384 is rejected with IBL_EINVAL.  Calls on different buffers
+ * may overlap.  A context without room for such a cluster (a small partition
+ * of a device) runs one block on a fixed array inside the library (16384 nodes
+ * x 9 doubles, 1.18 MB, held by every GPU that loads it until the process
+ * exits); there, calls whose executions overlap race on the array.  Make the
+ * first call in each context outside a stream capture (it asks for the
+ * cluster sizes).  Calls no allocating routine. */
 int ibl_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes, double alpha,
                            double gamma, double tol, int max_iter, int plus_sign, int32_t *result, void *stream);
+
+/* Tests only.  ibl_test_regularize_noalloc: ibl_regularize_noalloc as in a
+ * context whose widest cluster has `widest` blocks (16, 8 or 0 for none; else
+ * IBL_EINVAL); a wider one than the context takes fails at the launch.
+ * ibl_test_regularize_ctas (host only): blocks of the cluster that a mesh of
+ * n_nodes gets, 0 for the one-block kernel, where the question whether 16 (8)
+ * blocks fit is answered fits16 (fits8): 1 yes, 0 no, -1 could not be asked;
+ * *known (may be NULL) = 1 if that answer is kept for the context, else 0. */
+int ibl_test_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes, double alpha,
+                                double gamma, double tol, int max_iter, int plus_sign, int32_t *result, void *stream,
+                                int widest);
+int ibl_test_regularize_ctas(int n_nodes, int fits16, int fits8, int *known);
 
 /* The paper's trajectory loop with host buffers (Sec. 3.2, steps 1-4): for
  * each of n_frames frames, copy the frame (host, 9 doubles) to the device,

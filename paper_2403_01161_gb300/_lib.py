@@ -94,6 +94,10 @@ SIGNATURES = [
     ("ibl_regularize_now", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int)]),
     ("ibl_regularize_noalloc", ctypes.c_int, [_P, _P, _P, ctypes.c_int, ctypes.c_double, ctypes.c_double,
                                               ctypes.c_double, ctypes.c_int, ctypes.c_int, _P, _P]),
+    ("ibl_test_regularize_noalloc", ctypes.c_int, [_P, _P, _P, ctypes.c_int, ctypes.c_double, ctypes.c_double,
+                                                   ctypes.c_double, ctypes.c_int, ctypes.c_int, _P, _P, ctypes.c_int]),
+    ("ibl_test_regularize_ctas", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int,
+                                                ctypes.POINTER(ctypes.c_int)]),
     ("ibl_run_frames", ctypes.c_int, [_P, _P, _D, ctypes.c_int, ctypes.c_int, ctypes.POINTER(Observables)]),
     ("ibl_adjoint_workspace_size", ctypes.c_int, [_P, ctypes.c_longlong, ctypes.c_int, _SZ]),
     ("ibl_adjoint", ctypes.c_int, [_P, ctypes.c_longlong, ctypes.c_int, _P, ctypes.c_size_t, _D, _D, _D, _D]),

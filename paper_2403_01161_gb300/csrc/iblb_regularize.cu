@@ -1,13 +1,15 @@
 // iblb_regularize.cu -- mesh regularisation of Sec. 3.3 on a thread-block
 // cluster: the scheduled one of a droplet, the batched one of an ensemble,
-// and the allocation-free one on caller buffers; for meshes above 32768 nodes
-// the one-block kernel.
+// and the allocation-free one on caller buffers; for meshes above 32768 nodes,
+// and where the context has no room for such a cluster, one block.
 #include <cooperative_groups.h>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -17,10 +19,6 @@
 namespace iblb {
 namespace {
 
-// Mesh regularisation, Sec. 3.3, one block: x_o fixed, x_q the previous
-// iterate, x_p the new one (ping-pong between r and s1), x_b in s2.
-// patch_buf: patch buffer (parity) of the next step, rewritten from the
-// regularised positions.
 // This thread's share of the enclosed volume and of its first moment, summed
 // over signed tetrahedra (x_0, a, b, c) of the triangles, positions relative
 // to node 0: v[0] = V, v[1..3] = int (x - x_0) dV.
@@ -40,6 +38,66 @@ __device__ __forceinline__ void enclosed_volume_sums(const MeshView &M, double v
     }
 }
 
+// The iteration on one block: x_o fixed, x_q the previous iterate, x_p the new
+// one (ping-pong between r and s1), x_b in xb.  Leaves the result in r, returns
+// whether the exit test held.
+__device__ __forceinline__ bool regularize_block(double *r, double *xo, double *s1, double *xb, const int *nb_ptr,
+                                                 const int *nb_idx, const int nv, const RegParams &p, double *sh, int &it)
+{
+    double *buf[2] = {r, s1};
+    for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) xo[i] = r[i];
+    __syncthreads();
+    const double sg = p.plus_sign ? 1.0 : -1.0;
+    int cur = 0;
+    bool conv = false;
+    it = 0;
+    while (it < p.max_iter) {
+        ++it;
+        const double *xq = buf[cur];
+        double *xp = buf[cur ^ 1];
+        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+            const int b0 = nb_ptr[i], b1 = nb_ptr[i + 1];
+            const int ni = b1 - b0;
+            for (int a = 0; a < 3; ++a) {
+                double s = 0.0;
+                for (int k = b0; k < b1; ++k) s += xq[3 * nb_idx[k] + a];
+                const double v = p.alpha * xo[3 * i + a] + (1.0 - p.alpha) / ni * s;
+                xp[3 * i + a] = v;
+                xb[3 * i + a] = v - (p.alpha * xo[3 * i + a] + (1.0 - p.alpha) * xq[3 * i + a]);
+            }
+        }
+        __syncthreads();
+        double dmax = 0.0;
+        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+            const int b0 = nb_ptr[i], b1 = nb_ptr[i + 1];
+            const int ni = b1 - b0;
+            double d2 = 0.0;
+            for (int a = 0; a < 3; ++a) {
+                double s = 0.0;
+                for (int k = b0; k < b1; ++k) s += xb[3 * nb_idx[k] + a];
+                const double v = xp[3 * i + a] - (p.gamma * xb[3 * i + a] + sg * (1.0 - p.gamma) / ni * s);
+                xp[3 * i + a] = v;
+                const double d = v - xq[3 * i + a];
+                d2 += d * d;
+            }
+            dmax = fmax(dmax, sqrt(d2));
+        }
+        dmax = block_max(dmax, sh);  // includes a barrier after the writes above
+        cur ^= 1;
+        if (dmax < p.tol) {
+            conv = true;
+            break;
+        }
+    }
+    if (cur != 0) {
+        for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) r[i] = s1[i];
+    }
+    __syncthreads();
+    return conv;
+}
+
+// One block per mesh.  patch_buf: patch buffer (parity) of the next step,
+// rewritten from the regularised positions.
 __global__ void __launch_bounds__(1024) k_regularize(LbView L, MeshView M, RegParams p, int patch_buf)
 {
     __shared__ double sh[32];
@@ -73,55 +131,8 @@ __global__ void __launch_bounds__(1024) k_regularize(LbView L, MeshView M, RegPa
         block_sum<4>(v4, shv);
         V0 = v4[0];
     }
-    double *xo = M.s0, *xb = M.s2;
-    double *buf[2] = {M.r, M.s1};
-    for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) xo[i] = M.r[i];
-    __syncthreads();
-    const double sg = p.plus_sign ? 1.0 : -1.0;
-    int cur = 0, it = 0;
-    bool conv = false;
-    while (it < p.max_iter) {
-        ++it;
-        const double *xq = buf[cur];
-        double *xp = buf[cur ^ 1];
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = M.nb_ptr[i], b1 = M.nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xq[3 * M.nb_idx[k] + a];
-                const double v = p.alpha * xo[3 * i + a] + (1.0 - p.alpha) / ni * s;
-                xp[3 * i + a] = v;
-                xb[3 * i + a] = v - (p.alpha * xo[3 * i + a] + (1.0 - p.alpha) * xq[3 * i + a]);
-            }
-        }
-        __syncthreads();
-        double dmax = 0.0;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            const int b0 = M.nb_ptr[i], b1 = M.nb_ptr[i + 1];
-            const int ni = b1 - b0;
-            double d2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double s = 0.0;
-                for (int k = b0; k < b1; ++k) s += xb[3 * M.nb_idx[k] + a];
-                const double v = xp[3 * i + a] - (p.gamma * xb[3 * i + a] + sg * (1.0 - p.gamma) / ni * s);
-                xp[3 * i + a] = v;
-                const double d = v - xq[3 * i + a];
-                d2 += d * d;
-            }
-            dmax = fmax(dmax, sqrt(d2));
-        }
-        dmax = block_max(dmax, sh);  // includes a barrier after the writes above
-        cur ^= 1;
-        if (dmax < p.tol) {
-            conv = true;
-            break;
-        }
-    }
-    if (cur != 0) {
-        for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) M.r[i] = M.s1[i];
-    }
-    __syncthreads();
+    int it;
+    const bool conv = regularize_block(M.r, M.s0, M.s1, M.s2, M.nb_ptr, M.nb_idx, nv, p, sh, it);
     if (p.keep_volume) {
         // scale about the volume centroid back to the volume enclosed before
         double v4[4];
@@ -510,6 +521,24 @@ __global__ void __launch_bounds__(1024)
     regularize_body<true>(L, M, p, 0, P, cap, result);
 }
 
+// The allocation-free one on one block, for a context without room for a
+// cluster: x_o, the second iterate and x_b in a fixed array of the library
+// image, so that calls must not overlap.
+constexpr int kNoAllocMaxNodes = 16384;  // what one portable cluster's shared memory holds
+__device__ double g_noalloc_scratch[3][3 * kNoAllocMaxNodes];
+__global__ void __launch_bounds__(1024)
+    k_regularize_noalloc_block(double *r, const int *nb_ptr, const int *nb_idx, int nv, RegParams p, int *result)
+{
+    __shared__ double sh[32];
+    int it;
+    const bool conv = regularize_block(r, g_noalloc_scratch[0], g_noalloc_scratch[1], g_noalloc_scratch[2], nb_ptr, nb_idx,
+                                       nv, p, sh, it);
+    if (threadIdx.x == 0) {
+        result[0] = it;
+        result[1] = conv ? 1 : 0;
+    }
+}
+
 // Ensemble: the members of a group that are due, a cluster each (blockIdx.y
 // is the position among them).
 struct RegGroup {
@@ -554,42 +583,107 @@ cudaError_t launch_cluster(void (*k)(KArgs...), dim3 grid, int C, int P, cudaStr
     return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)..., P, reg_table(P));
 }
 
-}  // namespace
-
-// Whether the device takes a cluster of kRegCluster CTAs (one per SM).
-static bool big_cluster_ok()
+// Whether the current context takes a cluster of C such CTAs (one per SM): 1
+// yes, 0 no, -1 it could not be asked.
+int cluster_fits(int C)
 {
-    static int ok = -1;
-    if (ok < 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(kRegCluster);
-        cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = kRegSmemMax;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = kRegCluster;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        cudaError_t e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRegSmemMax);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_regularize_cluster, &cfg);
-        ok = e == cudaSuccess && n > 0 ? 1 : 0;
-        cudaGetLastError();  // a refusal only selects the portable cluster size
-    }
-    return ok == 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = kRegSmemMax;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    cudaError_t e = cudaSuccess;
+    if (C > 8) e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_regularize_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRegSmemMax);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_regularize_cluster, &cfg);
+    if (e == cudaSuccess) return n > 0 ? 1 : 0;
+    cudaGetLastError();  // a refusal only selects another form
+    return e == cudaErrorInvalidClusterSize || e == cudaErrorInvalidValue || e == cudaErrorNotSupported ? 0 : -1;
 }
+
+// CTAs of the widest cluster of the two sizes that `fits` grants, 0 for none;
+// `known` says whether that is the answer rather than a failure to ask.
+template <typename F>
+int widest_cluster(F &&fits, bool &known)
+{
+    known = true;
+    for (const int C : {kRegCluster, kRegClusterBatch}) {
+        const int f = fits(C);
+        if (f > 0) return C;
+        known = known && f == 0;
+    }
+    return 0;
+}
+
+// CTAs of the cluster for a mesh of nv nodes, 0: one block.
+int cluster_for(int nv, int widest) { return nv <= widest * kRegPerCta ? widest : 0; }
+
+// Id of the calling thread's current context (0 if there is none yet, or it
+// cannot be asked).
+unsigned long long context_id()
+{
+    using GetCurrent = CUresult (*)(CUcontext *);
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    const auto entry = [](const char *name) -> void * {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return q == cudaDriverEntryPointSuccess ? f : nullptr;
+    };
+    static void *const a = entry("cuCtxGetCurrent"), *const b = entry("cuCtxGetId");
+    if (!a || !b) return 0;
+    CUcontext c = nullptr;
+    unsigned long long id = 0;
+    if (reinterpret_cast<GetCurrent>(a)(&c) != CUDA_SUCCESS || !c) return 0;
+    return reinterpret_cast<GetId>(b)(c, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// widest_cluster of the current context, asked once per context: another
+// device, and a partition of one, is another context.
+int widest_cluster_here()
+{
+    struct Seen {
+        unsigned long long ctx;
+        int widest;
+    };
+    static std::mutex mu;
+    static Seen seen[16];
+    static unsigned next = 0;  // oldest entry
+    const unsigned long long ctx = context_id();
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        for (const Seen &s : seen)
+            if (ctx != 0 && s.ctx == ctx) return s.widest;
+    }
+    bool known = false;
+    const int w = widest_cluster(cluster_fits, known);
+    const unsigned long long now = context_id();  // asking creates the context if there was none
+    if (known && now != 0) {
+        std::lock_guard<std::mutex> lock(mu);
+        seen[next++ % 16] = Seen{now, w};
+    }
+    return w;
+}
+
+}  // namespace
 
 cudaError_t launch_regularize(const LbView &L, const MeshView &M, const RegParams &p, int buf, cudaStream_t s,
                               int prio)
 {
-    const int C = big_cluster_ok() ? kRegCluster : kRegClusterBatch;
-    if (M.nv > C * kRegPerCta) return launch_p(k_regularize, dim3(1), dim3(1024), s, prio, L, M, p, buf);
-    const int P = (M.nv + C - 1) / C;
-    return launch_cluster(k_regularize_cluster, dim3(C), C, P, s, prio, L, M, p, buf);
+    const int C = cluster_for(M.nv, widest_cluster_here());
+    if (C == 0) return launch_p(k_regularize, dim3(1), dim3(1024), s, prio, L, M, p, buf);
+    return launch_cluster(k_regularize_cluster, dim3(C), C, (M.nv + C - 1) / C, s, prio, L, M, p, buf);
 }
 
 // Up to six due members of a group take a 16-CTA cluster each, as a single
@@ -600,14 +694,14 @@ cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<c
 {
     static thread_local LbGroup lg;  // parameter blocks are large: kept off the stack
     static thread_local MeshGroup mg;
-    const int n = (int)E.lv.size();
+    const int n = (int)E.lv.size(), widest = widest_cluster_here();
     for (int m0 = 0; m0 < n; m0 += kGroup) {
         const int m1 = m0 + kGroup < n ? m0 + kGroup : n;
         RegGroup rg;
         int k = 0, nv_max = 0;
         for (int m = m0; m < m1; ++m) {
             if (!due[m]) continue;
-            if (E.mv[m].nv > kRegClusterBatch * kRegPerCta) {
+            if (E.mv[m].nv > kRegClusterBatch * kRegPerCta || widest == 0) {
                 const cudaError_t e = launch_regularize(E.lv[m], E.mv[m], params[m], buf, s, prio);
                 if (e != cudaSuccess) return e;
                 continue;
@@ -620,7 +714,7 @@ cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<c
             ++k;
         }
         if (k == 0) continue;
-        const int C = k <= 6 && big_cluster_ok() ? kRegCluster : kRegClusterBatch;
+        const int C = k <= 6 ? widest : kRegClusterBatch;
         const cudaError_t e = launch_cluster(k_regularize_batched, dim3(C, k), C, (nv_max + C - 1) / C, s, prio, lg, mg,
                                              rg, buf);
         if (e != cudaSuccess) return e;
@@ -632,28 +726,54 @@ cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<c
 
 // Allocation-free mesh regularisation: the cluster kernel on the caller's
 // positions and one-rings.  Its scratch is the cluster's shared memory, so
-// overlapping calls on different buffers do not disturb each other.  (Before,
-// one block with its scratch in a static device array: 1490 us for 10242
-// stretched and jittered nodes.)
-extern "C" int ibl_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes,
-                                      double alpha, double gamma, double tol, int max_iter, int plus_sign,
-                                      int32_t *result, void *stream)
+// overlapping calls on different buffers do not disturb each other.  One block
+// with its scratch in a static device array took 1490 us for 10242 stretched
+// and jittered nodes, against 117; it remains for a context without room for
+// a cluster.
+static int regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes, double alpha,
+                              double gamma, double tol, int max_iter, int plus_sign, int32_t *result, void *stream,
+                              int widest)
 {
     using namespace iblb;
     if (!r || !nb_ptr || !nb_idx || !result) return iblb_set_error(IBL_EINVAL, "null pointer argument");
-    constexpr int kMaxNodes = 16384;  // what one portable cluster's shared memory holds
-    static_assert(kMaxNodes <= kRegClusterBatch * kRegPerCta, "cluster capacity");
-    if (n_nodes < 1 || n_nodes > kMaxNodes)
+    static_assert(kNoAllocMaxNodes <= kRegClusterBatch * kRegPerCta, "cluster capacity");
+    if (n_nodes < 1 || n_nodes > kNoAllocMaxNodes)
         return iblb_set_error(IBL_EINVAL, "ibl_regularize_noalloc: n_nodes must be in 1..16384 (the size of its "
                                           "fixed scratch)");
     if (!(alpha >= 0 && alpha <= 1) || !(gamma >= 0 && gamma <= 1) || !(tol > 0) || max_iter < 1)
         return iblb_set_error(IBL_EINVAL, "regularisation parameters out of range");
     RegParams p{alpha, gamma, tol, max_iter, plus_sign ? 1 : 0};
-    const int C = big_cluster_ok() ? kRegCluster : kRegClusterBatch;
-    const cudaError_t e = launch_cluster(k_regularize_noalloc, dim3(C), C, (n_nodes + C - 1) / C,
-                                         static_cast<cudaStream_t>(stream), 0, r,
-                                         reinterpret_cast<const int *>(nb_ptr), reinterpret_cast<const int *>(nb_idx),
-                                         n_nodes, p, reinterpret_cast<int *>(result));
+    const int *ptr = reinterpret_cast<const int *>(nb_ptr), *idx = reinterpret_cast<const int *>(nb_idx);
+    int *res = reinterpret_cast<int *>(result);
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const int C = cluster_for(n_nodes, widest < 0 ? widest_cluster_here() : widest);
+    const cudaError_t e =
+        C == 0 ? launch_p(k_regularize_noalloc_block, dim3(1), dim3(1024), s, 0, r, ptr, idx, n_nodes, p, res)
+               : launch_cluster(k_regularize_noalloc, dim3(C), C, (n_nodes + C - 1) / C, s, 0, r, ptr, idx, n_nodes, p, res);
     if (e != cudaSuccess) return iblb_set_error(IBL_ECUDA, cudaGetErrorString(e));
     return IBL_OK;
+}
+
+extern "C" int ibl_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes,
+                                      double alpha, double gamma, double tol, int max_iter, int plus_sign,
+                                      int32_t *result, void *stream)
+{
+    return regularize_noalloc(r, nb_ptr, nb_idx, n_nodes, alpha, gamma, tol, max_iter, plus_sign, result, stream, -1);
+}
+
+extern "C" int ibl_test_regularize_noalloc(double *r, const int32_t *nb_ptr, const int32_t *nb_idx, int n_nodes,
+                                           double alpha, double gamma, double tol, int max_iter, int plus_sign,
+                                           int32_t *result, void *stream, int widest)
+{
+    if (widest != 0 && widest != iblb::kRegClusterBatch && widest != iblb::kRegCluster)
+        return iblb::iblb_set_error(IBL_EINVAL, "widest must be 0, 8 or 16");
+    return regularize_noalloc(r, nb_ptr, nb_idx, n_nodes, alpha, gamma, tol, max_iter, plus_sign, result, stream, widest);
+}
+
+extern "C" int ibl_test_regularize_ctas(int n_nodes, int fits16, int fits8, int *known)
+{
+    bool k = false;
+    const int w = iblb::widest_cluster([&](int C) { return C == iblb::kRegCluster ? fits16 : fits8; }, k);
+    if (known) *known = k ? 1 : 0;
+    return iblb::cluster_for(n_nodes, w);
 }
