@@ -851,10 +851,6 @@ int ensemble_layout(int n, ibl_lb *const *members, EnsembleLayout &L, std::strin
             why = "every member needs a lattice with a droplet mesh";
             return IBL_EINVAL;
         }
-        if ((long long)lb->v.n[0] * lb->v.n[1] >= (1LL << 22)) {
-            why = "an ensemble member's z plane exceeds 2^22 nodes";
-            return IBL_EINVAL;
-        }
         // the tables are sized for one tile per block, the most blocks there are
         lat[0] += lattice_blocks(lb, 128, 1);
         lat[1] += lattice_blocks(lb, 256, 1);
