@@ -400,8 +400,8 @@ int ibl_ensemble_step(ibl_ensemble *e, long long n);
 /* Launch shape of an ensemble step: IBL_ENSEMBLE_SHAPES candidates, shape
  * k = 8 c + 4 p + 2 t + w (c = 0..3).  The batched lattice update of the nodes outside
  * each droplet patch (almost all of a step's bytes) takes 128 (t = 0) or
- * 256 (t = 1) threads per block, each block updating that many consecutive
- * nodes of one z plane of one member, and prefetches the populations into
+ * 256 (t = 1) threads per block, a block updating runs of that many consecutive
+ * nodes of one member, and prefetches the populations into
  * L2 w resident waves of blocks ahead (w = 0 or 1).  p = 0 keeps the
  * droplet-side data (mesh, patch populations, force and velocity) in L2
  * with an evict_last policy, as a single droplet's step does; p = 1 uses the

@@ -187,8 +187,9 @@ __device__ __forceinline__ void bc_dispatch(T (&f)[19], const T (&uw)[3], int ru
 // ---------------------------------------------------------------------------
 // Lattice update: streaming (AA pattern) + boundary rebuild + moments with
 // half-force momentum + BGK + Guo source, Eqs. (LBMEQ)-(density_velocity_LB).
-// One thread per node; blocks tile (x, y) rows of one z plane, so no index
-// division is needed.  Indices are 32-bit (19 * stride < 2^31 is checked on
+// One thread per node: outside the patch consecutive nodes of the flattened
+// box, their coordinates by a division by constants (fast_div), in the patch
+// the rows of its box.  Indices are 32-bit (19 * stride < 2^31 is checked on
 // the host).  The collision works on opposite pairs (c_i, -c_i), whose
 // equilibrium and source terms share their even parts.
 // Node sets of one lattice launch: every node of a box without a droplet
@@ -1404,15 +1405,12 @@ __device__ __forceinline__ void interp_body(const LbView &L, const MeshView &M, 
 template <typename T, int LANES>
 __global__ void __launch_bounds__(128) k_interp(LbView L, MeshView M, int nblk)
 {
-    for (int b = blockIdx.x; b < nblk; b += (int)gridDim.x) {
-        interp_body<T, LANES>(L, M, b, nblk);
-        __syncthreads();  // the next pass reuses the body's shared rows
-    }
+    interp_body<T, LANES>(L, M, (int)blockIdx.x, nblk);
 }
 
 // Ensemble versions: block b works for member blk_member[b0 + b] as its
-// local block b0 + b - blk_start[member]; node-group kernels use ceil(nv/8)
-// blocks per member.
+// local block b0 + b - blk_start[member]; node-group kernels use ceil(nv /
+// kFwdNodesPerBlock) blocks per member.
 
 // The node groups b0 .. b0 + nb - 1 of a group of members, block-strided so
 // that a grid capped below nb leaves most SM slots to the concurrent
@@ -1766,7 +1764,7 @@ cudaError_t launch_lattice(const LbView &L, bool odd, bool record, int mode, int
 template <typename T, bool PER>
 static cudaError_t near_t(const LbView &L, bool odd, bool record, int pbuf, cudaStream_t s, int prio)
 {
-    const dim3 g(2 * 152), b(256);  // grid-stride over the patch box
+    const dim3 g(2 * sm_count()), b(256);  // grid-stride over the patch box
     if (odd) {
         if (record) return launch_p(k_lattice_near<T, true, true, PER>, g, b, s, prio, L, pbuf);
         return launch_p(k_lattice_near<T, true, false, PER>, g, b, s, prio, L, pbuf);

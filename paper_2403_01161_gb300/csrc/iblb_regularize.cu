@@ -687,8 +687,11 @@ cudaError_t launch_regularize(const LbView &L, const MeshView &M, const RegParam
 }
 
 // Up to six due members of a group take a 16-CTA cluster each, as a single
-// droplet does (the chip holds eight such clusters at once); more take 8 CTAs,
-// nineteen clusters at once.
+// droplet does; more take 8 CTAs.  The line is how many 16-CTA clusters run at
+// once beside the outside update, with one in hand for chips whose SMs are
+// grouped otherwise: us per step, regularised every other step, 2562 nodes
+// each, with 8 and 16 CTAs: 2 members 77.4 and 64.1, 6 124.3 and 110.7, 7
+// 137.0 and 123.1, 8 148.4 and 162.9 (the eighth waits), 12 190.8 and 205.3.
 cudaError_t launch_regularize_batched(const EnsembleView &E, const std::vector<char> &due,
                                       const std::vector<RegParams> &params, int buf, cudaStream_t s, int prio)
 {
