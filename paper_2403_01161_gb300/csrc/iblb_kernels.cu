@@ -1405,7 +1405,16 @@ __device__ __forceinline__ void interp_body(const LbView &L, const MeshView &M, 
 template <typename T, int LANES>
 __global__ void __launch_bounds__(128) k_interp(LbView L, MeshView M, int nblk)
 {
-    interp_body<T, LANES>(L, M, (int)blockIdx.x, nblk);
+    // The grid is one block per node group, so that this turns once; written
+    // straight, the same body compiled to a kernel that was slower in more
+    // boxes than it was faster (us per step, loop and straight: 24^3 FP64 21.7
+    // and 22.9, 96^3 regularised every tenth step 22.8 and 23.7, 128^3
+    // regularised every step 66.8 and 68.8; 32^3 FP64 32.7 and 32.1, 64^3 12.5
+    // and 12.3).
+    for (int b = blockIdx.x; b < nblk; b += (int)gridDim.x) {
+        interp_body<T, LANES>(L, M, b, nblk);
+        __syncthreads();
+    }
 }
 
 // Ensemble versions: block b works for member blk_member[b0 + b] as its
