@@ -958,7 +958,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1024 : 512) / NT)
 // member within the group), a warp per patch row as in k_lattice_near.  Capped
 // at 64 registers: at 80 its two blocks per SM held 62% of the register file
 // from the concurrent outside update for as long as they ran (step of 32
-// droplets 478 -> 457 us, of 16 centred ones 234 -> 223).
+// droplets 478 -> 457 us, of 16 centred ones 234 -> 223; 32 periodic ones 375
+// at 80, 358 at 64).  The odd form spills 16 bytes for it, 4 in periodic boxes.
 template <typename T, bool ODD, bool PER, class P>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lattice_near_batched(const __grid_constant__ LbGroup G,
                                                                                     const int buf)
