@@ -378,8 +378,8 @@ __device__ __forceinline__ void mirror_x(T (&g)[19], const bool on)
     });
 }
 
-// Offsets to a node's neighbours along each axis (odd step), in units of 1/S
-// node.  Periodic axes wrap.  On a Zou-He axis a missing neighbour points back
+// Offsets to a node's neighbours along each axis (odd step), S to a node (its
+// bytes, or 1).  Periodic axes wrap.  On a Zou-He axis a missing neighbour points back
 // at the node itself: a population whose source lies outside the box is an
 // unknown that the boundary rebuild overwrites before anything reads it, so
 // its load only needs an address inside the array, while a store to a missing
